@@ -554,8 +554,11 @@ int nchunks_for(oefe_ctx* c, int nv) {
   return std::max(1, std::min(1024, (4 * c->num_sms + pairs - 1) / pairs));
 }
 
+// M^oo -> (M^oo)^{-1} of the setup, in place, once per k-point. The one-CTA factor stays here: M^oo
+// is ill conditioned, so another order of its sums would change the stored operator's enrichment
+// rows in the ninth digit.
 template <typename S>
-int chol_inverse_t(oefe_ctx* c, S* A, int n, bool inverse, bool want_Linv, S* Y, int* info_host) {
+int chol_inverse_t(oefe_ctx* c, S* A, int n, bool inverse, S* Y, int* info_host) {
   OEFE_TRY(ensure_ws2(c, 256));
   int* d_info = c->d_status;
   OEFE_COUNTED k_chol<S><<<1, 1024, 0, c->stream>>>(A, n, d_info);
@@ -563,9 +566,9 @@ int chol_inverse_t(oefe_ctx* c, S* A, int n, bool inverse, bool want_Linv, S* Y,
   OEFE_CUDA_TRY(c, cudaMemcpyAsync(info_host, d_info, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   if (*info_host != 0) return OEFE_OK;
-  if (inverse || want_Linv) {
+  if (inverse) {
     OEFE_COUNTED k_trinv<S><<<(n + 127) / 128, 128, 0, c->stream>>>(A, Y, n);
-    if (inverse) OEFE_COUNTED k_yhy<S><<<(n * n + 255) / 256, 256, 0, c->stream>>>(Y, A, n);
+    OEFE_COUNTED k_yhy<S><<<(n * n + 255) / 256, 256, 0, c->stream>>>(Y, A, n);
     OEFE_CUDA_TRY(c, cudaGetLastError());
   }
   return OEFE_OK;
@@ -590,13 +593,16 @@ int orthonormalize_t(oefe_ctx* c, int ik, S* X, int nv, int ld, double* cond) {
   const size_t sbytes = (((size_t)nv * nv * sizeof(S) + 255) / 256) * 256;
   const size_t pbytes = (size_t)nchunk * nv * nv * sizeof(S);
   const size_t pbytes_a = ((pbytes + 255) / 256) * 256;
-  OEFE_TRY(ensure_ws(c, wbytes + 2 * sbytes + pbytes_a + (size_t)nv * sizeof(double)));
+  const size_t dbytes = (((size_t)nv * sizeof(double) + 255) / 256) * 256;
+  OEFE_TRY(ensure_ws(c, wbytes + 3 * sbytes + pbytes_a + dbytes + chol_scratch(nv, sizeof(S))));
   char* base = (char*)c->ws;
   S* W = (S*)base;
   S* Sm = (S*)(base + wbytes);
   S* Y = (S*)(base + wbytes + sbytes);
   S* part = (S*)(base + wbytes + 2 * sbytes);
   double* dsc = (double*)(base + wbytes + 2 * sbytes + pbytes_a);
+  S* Lm = (S*)(base + wbytes + 2 * sbytes + pbytes_a + dbytes);
+  void* cscr = base + wbytes + 3 * sbytes + pbytes_a + dbytes;
   for (int pass = 0; pass < 2; ++pass) {
     OEFE_TRY(apply_M<S>(c, K, X, ld, nv, W, nv));
     OEFE_TRY(gram<S>(c, X, ld, W, nv, n, nv, Sm, part, nchunk));
@@ -611,14 +617,14 @@ int orthonormalize_t(oefe_ctx* c, int ik, S* X, int nv, int ld, double* cond) {
       OEFE_CUDA_TRY(c, cudaGetLastError());
     }
     int info = 0;
-    OEFE_TRY(chol_inverse_t<S>(c, Sm, nv, false, true, Y, &info));
+    OEFE_TRY(chol_factor_inverse<S>(c, Sm, Lm, Y, nv, cscr, c->d_status + 3, &info));
     if (info != 0) {
       c->err = "orthonormalize: Gram matrix not positive definite at column " + std::to_string(info);
       return OEFE_ERR_CHOLESKY;
     }
     if (pass == 0 && cond) {
       std::vector<S> Lh((size_t)nv * nv);
-      OEFE_CUDA_TRY(c, cudaMemcpyAsync(Lh.data(), Sm, Lh.size() * sizeof(S), cudaMemcpyDeviceToHost, c->stream));
+      OEFE_CUDA_TRY(c, cudaMemcpyAsync(Lh.data(), Lm, Lh.size() * sizeof(S), cudaMemcpyDeviceToHost, c->stream));
       OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
       double mx = 0, mn = 1e300;
       for (int i = 0; i < nv; ++i) {
@@ -688,8 +694,8 @@ int chol_inverse_inplace(oefe_ctx* c, double* A, int n, bool cplx, bool inverse,
   if (n == 0) { *info_host = 0; return OEFE_OK; }
   const size_t sb = cplx ? sizeof(cd) : sizeof(double);
   OEFE_TRY(ensure_ws2(c, (size_t)n * n * sb + 256));
-  if (cplx) return chol_inverse_t<cd>(c, (cd*)A, n, inverse, false, (cd*)c->ws2, info_host);
-  return chol_inverse_t<double>(c, A, n, inverse, false, (double*)c->ws2, info_host);
+  if (cplx) return chol_inverse_t<cd>(c, (cd*)A, n, inverse, (cd*)c->ws2, info_host);
+  return chol_inverse_t<double>(c, A, n, inverse, (double*)c->ws2, info_host);
 }
 
 int orthonormalize(oefe_ctx* c, int ik, void* X, int nv, int ld, int dtype, double* cond) {

@@ -253,6 +253,11 @@ int build_hamiltonian(oefe_ctx* c, const double* veff, int store);
 // dense helpers (linalg.cu)
 int chol_inverse_inplace(oefe_ctx* c, double* A, int n, bool cplx, bool inverse, int* info_host);
 
+// blocked Cholesky factor and triangular inverse (chol.cu)
+size_t chol_scratch(int n, size_t scalar);
+template <typename S>
+int chol_factor_inverse(oefe_ctx* c, S* A, S* L, S* Y, int n, void* scratch, int* d_info, int* info_host);
+
 // operator application and filter (filter.cu)
 int apply_op(oefe_ctx* c, int ik, const void* X, void* Y, int nv, int ld, int dtype, bool minv);
 int apply_op2(oefe_ctx* c, int ik, const void* X, int ldx, void* Y, int ldy, int nv, int dtype, bool minv);
