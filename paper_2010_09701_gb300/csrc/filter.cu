@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(CWARPS * 32) k_cell_apply(const typename Sc<T,
                                                             const int* __restrict__ act_off,
                                                             const int* __restrict__ act_idx, int nloc, int npad,
                                                             int64_t nh, typename Sc<T, C>::type* __restrict__ Z,
-                                                            const int* __restrict__ cells, int compact) {
+                                                            const int* __restrict__ cells, int compact, int rpc) {
   using S = typename Sc<T, C>::type;
   extern __shared__ unsigned char smem_raw[];
   S* Xs = reinterpret_cast<S*>(smem_raw);  // npad x NB
@@ -67,7 +67,8 @@ __global__ void __launch_bounds__(CWARPS * 32) k_cell_apply(const typename Sc<T,
   }
   __syncthreads();
   const S* He = H + hslot * npad * npad;
-  for (int r = warp; r < naug; r += CWARPS) {
+  const int r_end = min(naug, ((int)blockIdx.z + 1) * rpc);   // this CTA's rows
+  for (int r = blockIdx.z * rpc + warp; r < r_end; r += CWARPS) {
     const S* hr = He + (size_t)r * npad;
     S acc = Sc<T, C>::zero();
     for (int k0 = 0; k0 < naug; k0 += 32) {
@@ -99,7 +100,7 @@ __global__ void __launch_bounds__(CWARPS * 32) k_cell_apply_z3(const cd* __restr
                                                               const int* __restrict__ act_off,
                                                               const int* __restrict__ act_idx, int nloc, int npad,
                                                               int64_t nh, cd* __restrict__ Z,
-                                                              const int* __restrict__ cells, int compact) {
+                                                              const int* __restrict__ cells, int compact, int rpc) {
   extern __shared__ unsigned char smem_raw[];
   double* Xr = reinterpret_cast<double*>(smem_raw);  // npad x NB3 each
   double* Xi = Xr + (size_t)npad * NB3;
@@ -124,9 +125,10 @@ __global__ void __launch_bounds__(CWARPS * 32) k_cell_apply_z3(const cd* __restr
   }
   __syncthreads();
   const cd* He = H + hslot * npad * npad;
-  for (int r0 = 2 * warp; r0 < naug; r0 += 2 * CWARPS) {
+  const int r_end = min(naug, ((int)blockIdx.z + 1) * rpc);   // this CTA's rows
+  for (int r0 = blockIdx.z * rpc + 2 * warp; r0 < r_end; r0 += 2 * CWARPS) {
     const int r = r0 + half;
-    const bool rv = r < naug;
+    const bool rv = r < r_end;
     const cd* hr = He + (size_t)(rv ? r : r0) * npad;
     double p1 = 0.0, p2 = 0.0, p3 = 0.0;
     for (int k0 = 0; k0 < naug; k0 += 16) {
@@ -569,6 +571,17 @@ struct Step {
   double alpha, cshift, beta;
 };
 
+// Rows per CTA of the dense cell products: a CTA takes every row of its cell and vector block when
+// those blocks fill the GPU twice over, else the rows are shared out (multiples of 16, one pass of
+// the warps) until they do. Each row's sum is the same either way. The two-atom cell has 16 refined
+// cells, so 16 CTAs: 183 us a product of 20 real vectors, 757 us of 13 complex ones.
+int dense_rows_per_cta(const oefe_ctx* c, long long blocks) {
+  const int most = (c->npad + 15) / 16;
+  const long long want = (2LL * c->num_sms + blocks - 1) / std::max(blocks, 1LL);
+  const int nz = (int)std::max(1LL, std::min<long long>(want, most));
+  return ((c->npad + nz - 1) / nz + 15) / 16 * 16;
+}
+
 template <typename T, bool C>
 int launch_step(oefe_ctx* c, const KData& K, int dtype, const void* Hm, const void* Xin, int ldin, int nv, const Step& st,
                 const void* Xk, int ldk, const void* Xm1, int ldm1, void* Y, int ldy, void* Zbuf, cd* Yo, bool mma) {
@@ -586,22 +599,24 @@ int launch_step(oefe_ctx* c, const KData& K, int dtype, const void* Hm, const vo
   } else if (ndense == 0) {
     // every cell was a single-leaf cell
   } else if (sizeof(T) == 8 && C) {
-    dim3 grid(ndense, (nv + NB3 - 1) / NB3);
+    const int vb = (nv + NB3 - 1) / NB3, rpc = dense_rows_per_cta(c, (long long)ndense * vb);
+    dim3 grid(ndense, vb, (c->npad + rpc - 1) / rpc);
     const size_t smem = (size_t)c->npad * NB3 * 3 * sizeof(double);
     if (smem > 227 * 1024) { c->err = "cell matrices too large for the shared-memory gather"; return OEFE_ERR_ARG; }
     OEFE_CUDA_TRY(c, cudaFuncSetAttribute(k_cell_apply_z3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     OEFE_COUNTED k_cell_apply_z3<<<grid, CWARPS * 32, smem, c->stream>>>((const cd*)Hm, (const cd*)Xin, ldin, nv,
                                                                         c->d_cell_nodes, c->d_act_off, c->d_act_idx,
                                                                         c->nloc, c->npad, c->nh, (cd*)Zbuf, dense_cells,
-                                                                        compact);
+                                                                        compact, rpc);
   } else {
-    dim3 grid(ndense, (nv + NB - 1) / NB);
+    const int vb = (nv + NB - 1) / NB, rpc = dense_rows_per_cta(c, (long long)ndense * vb);
+    dim3 grid(ndense, vb, (c->npad + rpc - 1) / rpc);
     const size_t smem = (size_t)c->npad * NB * sizeof(S);
     if (smem > 227 * 1024) { c->err = "cell matrices too large for the shared-memory gather"; return OEFE_ERR_ARG; }
     OEFE_CUDA_TRY(c, cudaFuncSetAttribute(k_cell_apply<T, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     OEFE_COUNTED k_cell_apply<T, C><<<grid, CWARPS * 32, smem, c->stream>>>((const S*)Hm, (const S*)Xin, ldin, nv, c->d_cell_nodes,
                                                                c->d_act_off, c->d_act_idx, c->nloc, c->npad, c->nh,
-                                                               (S*)Zbuf, dense_cells, compact);
+                                                               (S*)Zbuf, dense_cells, compact, rpc);
   }
   if ((c->timing >> dtype) & 1) cudaEventRecord(timing_event(c), c->stream);
   const int64_t tot = c->nh * nv;
