@@ -16,7 +16,7 @@
 
 static void free_all(oefe_ctx* c) {
   for (auto& K : c->kd) {
-    dev_free(K.gamma); dev_free(K.Moo); dev_free(K.Mooinv); dev_free(K.H64); dev_free(K.H32); dev_free(K.Hbf); dev_free(K.rexp);
+    dev_free(K.gamma); dev_free(K.Moo); dev_free(K.Mooinv); dev_free(K.H64); dev_free(K.H32); dev_free(K.Hbf); dev_free(K.Hp);
     dev_free(K.E0); dev_free(K.NO); dev_free(K.NOp);
   }
   c->kd.clear();
@@ -39,8 +39,6 @@ static void free_all(oefe_ctx* c) {
   dev_free(c->d_dense_cells);
   dev_free(c->d_sf_index);
   dev_free(c->d_dense_index);
-  dev_free(c->d_oz_jobs);
-  dev_free(c->d_oz_jobs_c);
   dev_free(c->d_rotp);
   c->d_rotp = nullptr;
   c->rotp_bytes = 0;

@@ -866,16 +866,17 @@ __global__ void k_hermitize(S* A, int n) {
   }
 }
 
-// Where a finished OEFE cell matrix goes: the FP64 / FP32 / bf16-split copies, or (the
+// Where a finished OEFE cell matrix goes: the FP64 / FP32 / FP32-pair / bf16-split copies, or (the
 // setup pass of the V-independent part) only its CO and OO blocks into the per-cell cache E0
 // (CO: nloc x ne_max, then OO: ne_max x ne_max).
 struct StoreOut {
   void* H64;
   void* H32;
   __nv_bfloat16* Hbf;
+  float* Hp;
   int parts, nloc, npad, ne_max;
   cd* E0;
-  // compact layout of H64 (KData::compact): cell -> dense-list position or sum-factorization
+  // compact layout of H64 / Hp (KData::compact): cell -> dense-list position or sum-factorization
   // row, and where the strips start
   const int* dense_index;
   const int* sf_index;
@@ -883,7 +884,7 @@ struct StoreOut {
   int compact;
 };
 
-// v in FP64 and as FP32 pairs (pr, pi): the three-part bf16 split is taken from the pairs
+// v in FP64 and as FP32 pairs (pr, pi): the pair copy and the bf16 splits are taken from the pairs
 template <typename S>
 __device__ inline void store_entry2(const StoreOut& O, int e, int ne, int r, int c, cd v, f2 pr, f2 pi) {
   const int nloc = O.nloc, npad = O.npad;
@@ -895,7 +896,7 @@ __device__ inline void store_entry2(const StoreOut& O, int e, int ne, int r, int
     return;
   }
   const size_t o = (size_t)e * npad * npad + (size_t)r * npad + c;
-  // H64 offset: the full layout, or the compact one (the CFE-CFE block of single-leaf cells and
+  // H64 / Hp offset: the full layout, or the compact one (the CFE-CFE block of single-leaf cells and
   // rows beyond the enrichment strip are not kept)
   long long oc = (long long)o;
   if (O.compact) {
@@ -911,9 +912,11 @@ __device__ inline void store_entry2(const StoreOut& O, int e, int ne, int r, int
   if constexpr (sizeof(S) == sizeof(cd)) {
     if (O.H64 && oc >= 0) reinterpret_cast<cd*>(O.H64)[oc] = v;
     if (O.H32) reinterpret_cast<cf*>(O.H32)[o] = cf{(float)v.x, (float)v.y};
+    if (O.Hp && oc >= 0) reinterpret_cast<float4*>(O.Hp)[oc] = make_float4(pr.h, pr.l, pi.h, pi.l);
   } else {
     if (O.H64 && oc >= 0) reinterpret_cast<double*>(O.H64)[oc] = v.x;
     if (O.H32) reinterpret_cast<float*>(O.H32)[o] = (float)v.x;
+    if (O.Hp && oc >= 0) reinterpret_cast<float2*>(O.Hp)[oc] = make_float2(pr.h, pr.l);
   }
   if (O.Hbf) {
     // tile-contiguous: per cell [K tile of 64 columns][M tile of 128 rows][plane][128][64], so that
@@ -952,7 +955,7 @@ __device__ inline void store_entry2(const StoreOut& O, int e, int ne, int r, int
 
 template <typename S>
 __device__ inline void store_entry(const StoreOut& O, int e, int ne, int r, int c, cd v) {
-  const bool need = O.Hbf && O.parts == 3;
+  const bool need = O.Hp || (O.Hbf && O.parts == 3);
   store_entry2<S>(O, e, ne, r, c, v, need ? f2_from(v.x) : f2{0.0f, 0.0f}, need ? f2_from(v.y) : f2{0.0f, 0.0f});
 }
 
@@ -1366,6 +1369,7 @@ static int run_cell_kernel(oefe_ctx* c, KData& K, int mode, const double* veff, 
     O.H64 = (store & OEFE_STORE_F64) ? K.H64 : nullptr;
     O.H32 = (store & OEFE_STORE_F32) ? K.H32 : nullptr;
     O.Hbf = (store & (OEFE_STORE_BF16X3 | OEFE_STORE_BF16X6)) ? (__nv_bfloat16*)K.Hbf : nullptr;
+    O.Hp = (store & OEFE_STORE_F64PAIR) ? K.Hp : nullptr;
     O.parts = K.bf_parts;
     O.nloc = c->nloc;
     O.npad = c->npad;
@@ -1385,7 +1389,7 @@ static int run_cell_kernel(oefe_ctx* c, KData& K, int mode, const double* veff, 
     }
     if (mode == 0) {
       // the V-independent OEFE blocks CO0, OO0 of each cell into the cache
-      O = StoreOut{nullptr, nullptr, nullptr, 0, c->nloc, c->npad, c->ne_max, (cd*)K.E0, nullptr, nullptr, 0, 0, 0};
+      O = StoreOut{nullptr, nullptr, nullptr, nullptr, 0, c->nloc, c->npad, c->ne_max, (cd*)K.E0, nullptr, nullptr, 0, 0, 0};
       TransformSf T;
       T.sf = c->use_sumfac && c->n_sf > 0 ? c->d_sf : nullptr;
       T.sf_index = c->d_sf_index;
@@ -1422,7 +1426,7 @@ int setup_kpoints(oefe_ctx* c, int nk, const double* k, const double* w) {
   if (!c->has_quad) { c->err = "kpoints: call oefe_quadrature first"; return OEFE_ERR_STATE; }
   if (nk < 1 || nk > 4096 || !k || !w) { c->err = "kpoints: need 1 <= nk <= 4096, k, w"; return OEFE_ERR_ARG; }
   for (auto& K : c->kd) {
-    dev_free(K.gamma); dev_free(K.Moo); dev_free(K.Mooinv); dev_free(K.H64); dev_free(K.H32); dev_free(K.Hbf); dev_free(K.rexp);
+    dev_free(K.gamma); dev_free(K.Moo); dev_free(K.Mooinv); dev_free(K.H64); dev_free(K.H32); dev_free(K.Hbf); dev_free(K.Hp);
     dev_free(K.E0); dev_free(K.NO); dev_free(K.NOp);
   }
   c->kd.assign(nk, KData());
@@ -1541,13 +1545,16 @@ int build_hamiltonian(oefe_ctx* c, const double* veff, int store) {
       if (*p) return OEFE_OK;
       return dev_alloc(c, p, bytes);
     };
-    if (compact != K.compact) {   // another layout: a new FP64 buffer
+    if (compact != K.compact) {   // another layout: new FP64 / pair buffers
       dev_free(K.H64);
+      dev_free(K.Hp);
       K.H64 = nullptr;
+      K.Hp = nullptr;
     }
     K.compact = compact;
     st = keep((void**)&K.H64, store & OEFE_STORE_F64, n64 * sb);
     if (st == OEFE_OK) st = keep((void**)&K.H32, store & OEFE_STORE_F32, n * sb / 2);
+    if (st == OEFE_OK) st = keep((void**)&K.Hp, store & OEFE_STORE_F64PAIR, n64 * sb);
     const int parts = (store & OEFE_STORE_BF16X6) ? 3 : (store & OEFE_STORE_BF16X3) ? 2 : 0;
     if (parts != K.bf_parts) {   // a different split: a new buffer
       dev_free(K.Hbf);
@@ -1557,9 +1564,6 @@ int build_hamiltonian(oefe_ctx* c, const double* veff, int store) {
     if (st == OEFE_OK) st = keep(&K.Hbf, parts > 0, n * sb / 4 * parts);
     if (st == OEFE_OK && c->nO > 0) st = ensure_orth_enrichment(c, K);
     if (st == OEFE_OK) st = run_cell_kernel(c, K, 2, veff, d_gw, nullptr, nullptr, store);
-    // pair products: the tensor-core dense blocks take one exponent per matrix row
-    K.pairs = (store & OEFE_STORE_F64PAIR) != 0;
-    if (st == OEFE_OK && K.pairs) st = oz_operator_ready(c, K);
     if (st != OEFE_OK) break;
     K.built = true;
   }

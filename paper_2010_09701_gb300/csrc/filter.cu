@@ -589,9 +589,8 @@ int launch_step(oefe_ctx* c, const KData& K, int dtype, const void* Hm, const vo
   if ((c->timing >> dtype) & 1) cudaEventRecord(timing_event(c), c->stream);
   // FP64: single-leaf cells by sum factorization, the others dense
   const bool sf = sizeof(T) == 8 && sumfac_ready(c);
-  const bool oz = sf && c->f64_products == OEFE_F64_PAIRS;   // pair mode: the dense cells on the tensor cores
   const int* dense_cells = sf ? c->d_dense_cells : nullptr;
-  const int ndense = oz ? 0 : sf ? c->n_dense : c->ncells;
+  const int ndense = sf ? c->n_dense : c->ncells;
   const int compact = (sizeof(T) == 8 && K.compact) ? 1 : 0;
   if (compact && !sf) { c->err = "compact FP64 storage needs the sum-factorized products"; return OEFE_ERR_STATE; }
   if (sf) OEFE_TRY(launch_cell_apply_sf(c, K, Xin, ldin, nv, C, Zbuf, c->stream));
@@ -666,20 +665,6 @@ int check_apply_args(oefe_ctx* c, int ik, const void* X, int nv, int ld, int dty
 
 }  // namespace
 
-// End of an operator application: wait, and in pair mode read the tensor-core kernels' error word
-static int finish_apply(oefe_ctx* c, int dtype) {
-  int flag = 0;
-  const bool oz = dtype_fp64(dtype) && c->f64_products == OEFE_F64_PAIRS;
-  if (oz) OEFE_CUDA_TRY(c, cudaMemcpyAsync(&flag, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  if (flag) {
-    cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
-    c->err = "operator application: a tensor-core wait timed out";
-    return OEFE_ERR_TIMEOUT;
-  }
-  return OEFE_OK;
-}
-
 // vectors per pass of the operator application: the per-cell products of one pass are held at once
 // (ncells x npad x chunk scalars), so wide blocks go through in column chunks
 constexpr int APPLY_CHUNK = 64;
@@ -699,7 +684,8 @@ int apply_op2(oefe_ctx* c, int ik, const void* X, int ldx, void* Y, int ldy, int
     OEFE_TRY(dispatch_step(c, c->kd[ik], dtype, (const char*)X + (size_t)c0 * es, ldx, nvc, st, nullptr, 0, nullptr, 0,
                            (char*)Y + (size_t)c0 * es, ldy, base, (cd*)(base + zbytes)));
   }
-  return finish_apply(c, dtype);
+  OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  return OEFE_OK;
 }
 
 int apply_op(oefe_ctx* c, int ik, const void* X, void* Y, int nv, int ld, int dtype, bool minv) {
@@ -723,7 +709,8 @@ int apply_op_scratch(oefe_ctx* c, int ik, const void* X, int ldx, void* Y, int l
   char* base = (char*)scratch;
   Step st{minv ? 1 : 0, 1.0, 0.0, 0.0};
   OEFE_TRY(dispatch_step(c, c->kd[ik], dtype, X, ldx, nv, st, nullptr, 0, nullptr, 0, Y, ldy, base, (cd*)(base + zbytes)));
-  return finish_apply(c, dtype);
+  OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  return OEFE_OK;
 }
 
 // Y = M^{-1} H X for one low-precision column through the tensor-core products
@@ -836,7 +823,7 @@ int cheb_filter(oefe_ctx* c, int ik, void* X, int nv, int ld, int dtype, int deg
                                        cudaMemcpyDeviceToDevice, c->stream));
   }
   OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  if (mma || c->f64_products == OEFE_F64_PAIRS) {
+  if (mma) {
     int flag = 0;
     OEFE_CUDA_TRY(c, cudaMemcpy(&flag, c->d_status, sizeof(int), cudaMemcpyDeviceToHost));
     if (flag) {

@@ -74,9 +74,8 @@ struct KData {
   double* Mooinv = nullptr;  // nO x nO scalars (FP64)
   double* H64 = nullptr;     // (ncells, npad, npad) scalars
   float* H32 = nullptr;      // (ncells, npad, npad) float or cf
-  bool pairs = false;        // built with OEFE_STORE_F64PAIR
-  int* rexp = nullptr;       // largest exponent of every row of the dense blocks (cell_oz.cu)
-  // H64 in the compact layout (OEFE_STORE_COMPACT): the cells with several quadrature leaves
+  float* Hp = nullptr;       // (ncells, npad, npad) FP64 values as FP32 pairs (h, l per real part)
+  // H64 / Hp in the compact layout (OEFE_STORE_COMPACT): the cells with several quadrature leaves
   // whole (npad x npad each, in the order of the dense-cell list), then per single-leaf cell (in the
   // order of the sum-factorization list) its enrichment strip: the CO block (nloc x ne_max), then
   // the enrichment rows (ne_max x npad); the CFE-CFE block of those cells is not stored (their
@@ -198,7 +197,7 @@ struct oefe_ctx {
   // sum-factorized FP64 products on single-leaf cells (sumfac.cu)
   int use_sumfac = 1;
   int f64_products = OEFE_F64_NATIVE;   // arithmetic of the sum-factorized FP64 products
-  int sf_variant = -1;                  // launch shape of the general pair product (-1: the default, 2)
+  int sf_variant = -1;                  // launch shape of the pair product: chosen by timing at first use
   int fields_variant = -1;              // pass width of the pair fields: chosen by timing at first use
   double* d_sf = nullptr;               // per single-leaf cell: n1, 1D tables, M/K/A
   int* d_sf_cells = nullptr;            // single-leaf cells
@@ -206,10 +205,6 @@ struct oefe_ctx {
   int* d_sf_index = nullptr;            // cell -> row of d_sf, or -1
   int* d_dense_index = nullptr;         // cell -> position in d_dense_cells, or -1
   int n_sf = 0, n_dense = 0, sf_nbuf = 0;
-  std::vector<int> sf_cells_h, dense_cells_h, sf_n1_h;   // host copies of the two lists; points per axis
-  void* d_oz_jobs = nullptr;            // tensor-core dense blocks: job tables, full and compact layout
-  void* d_oz_jobs_c = nullptr;
-  int n_oz_jobs = 0;
   double* d_veff = nullptr;             // V_eff at the points of the last operator build
   int tune_merge = -1;                  // TMA kernel: merged real-part MMAs (1), separate (0), untuned (-1)
   double tune_ms[6] = {0, 0, 0, 0, 0, 0};
@@ -298,11 +293,6 @@ size_t cell_mma_smem(bool cplx, int nb);
 // sum factorization (sumfac.cu)
 int setup_sumfac(oefe_ctx* c);
 bool sumfac_ready(const oefe_ctx* c);
-int launch_sf_cc(oefe_ctx* c, const KData& K, const void* X, int ldx, int nv, bool cplx, void* Z, int first, int count,
-                 int n1, bool* done, cudaStream_t st);
-// dense blocks of the pair products on the tensor cores (cell_oz.cu)
-int oz_operator_ready(oefe_ctx* c, KData& K);
-int launch_cell_oz(oefe_ctx* c, const KData& K, const void* X, int ldx, int nv, bool cplx, void* Z, cudaStream_t st);
 int launch_cell_apply_sf(oefe_ctx* c, const KData& K, const void* X, int ldx, int nv, bool cplx, void* Z,
                          cudaStream_t st);
 void cell_box(const oefe_ctx* c, int e, double lo[3], double hi[3]);
@@ -337,7 +327,7 @@ int band_trace(oefe_ctx* c, int ik, const void* X, int nv, int ld, int dtype, do
 int band_trace_vjp(oefe_ctx* c, int ik, const void* X, int nv, int ld, int dtype, double alpha, double* gV, void* gX);
 int apply_h_vjp(oefe_ctx* c, int ik, const void* X, const void* Gy, double* gV, void* gX, int nv, int ld, int dtype);
 
-// compact layout of the FP64 cell matrices: scalars of one enrichment strip, and of the
+// compact layout of the FP64 / FP32-pair cell matrices: scalars of one enrichment strip, and of the
 // whole store (see KData::compact)
 inline size_t compact_strip(const oefe_ctx* c) { return (size_t)c->nloc * c->ne_max + (size_t)c->ne_max * c->npad; }
 inline size_t h64_entries(const oefe_ctx* c, bool compact) {

@@ -45,8 +45,8 @@ void lagrange_host(const std::vector<double>& xn, double x, double* L, double* D
 struct SfArgs {
   const double* sf;          // per listed cell: SF_STRIDE doubles
   const int* cells;          // listed cells
-  int count;
   const void* H;             // FP64 cell matrices (npad x npad per cell, or the compact layout)
+  const float* Hp;           // the same as FP32 pairs (h, l per real part), for V = f2
   int compact, ne_max;       // compact layout: the listed cell's strip starts at sf_base + slot * strip
   long long sf_base, strip;
   const void* X;
@@ -156,14 +156,93 @@ __global__ void __launch_bounds__(NT) k_cell_apply_sf(const SfArgs A) {
       else Z[((size_t)e * npad + r) * A.nv + v0 + v] = yr;
     }
   } else {
-    // pairs: the enrichment blocks are in Z already (cell_oz.cu); the node rows are added
-    for (int t = threadIdx.x; t < nloc * NV; t += NT) {
-      const int v = t % NV, r = t / NV;
+    // one item per thread, all NV vectors: each pair of the matrix is loaded once for NV * R
+    // independent accumulations. Items: a node row over the ne enrichment columns, or a chunk of
+    // at most EC columns of an enrichment row (the partial sums meet in shared memory), so that
+    // the items have about the same length.
+    int nch = min((naug + 47) / 48, A.nbuf / max(ne, 1));  // chunks of about 48 columns; the
+    nch = max(nch, 1);                                      // partial sums must fit in Ab
+    const int EC = (naug + nch - 1) / nch;
+    V* part = Ab;                                          // (ne * nch) x J partial sums
+    for (int it = threadIdx.x; it < nloc + ne * nch; it += NT) {
+      int r, ca, cb, pidx = 0;
+      if (it < nloc) {
+        r = it;
+        ca = nloc;
+        cb = naug;
+      } else {
+        // consecutive items take the same chunk of consecutive enrichment rows, so that a warp reads
+        // one row of the vectors per column (a broadcast) instead of one per chunk (chunks a multiple
+        // of 128 bytes apart fall in the same banks)
+        const int q = it - nloc, ch = q / ne, i = q % ne;
+        r = nloc + i;
+        ca = ch * EC;
+        cb = min(naug, ca + EC);
+        pidx = i * nch + ch;
+      }
+      Acc y[J];
+#pragma unroll
+      for (int j = 0; j < J; ++j) {
+        const V s = it < nloc ? Ys[(size_t)r * J + j] : v_from<V>(0.0);
+        y[j] = Acc{s.h, s.l};
+      }
+      if constexpr (CPLX) {
+        int cf = 0;
+        const long long ro = sf_row(A, e, blockIdx.y, r, &cf);
+        const float4* hr = reinterpret_cast<const float4*>(A.Hp) + ro - cf;   // hr[c] for c >= cf
+        float4 hn = ca < cb ? hr[ca] : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int cidx = ca; cidx < cb; ++cidx) {
+          const float4 h = hn;
+          if (cidx + 1 < cb) hn = hr[cidx + 1];     // next pair in flight during the products
+          const V hre{h.x, h.y}, him{h.z, h.w}, nhim = v_neg(him);
+          const V* x = Xs + (size_t)cidx * J;
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            const V xr = x[2 * v], xi = x[2 * v + 1];
+            v_mac(y[2 * v], hre, xr);
+            v_mac(y[2 * v + 1], hre, xi);
+            v_mac(y[2 * v], nhim, xi);
+            v_mac(y[2 * v + 1], him, xr);
+          }
+        }
+      } else {
+        int cf = 0;
+        const long long ro = sf_row(A, e, blockIdx.y, r, &cf);
+        const float2* hr = reinterpret_cast<const float2*>(A.Hp) + ro - cf;   // hr[c] for c >= cf
+        float2 hn = ca < cb ? hr[ca] : make_float2(0.f, 0.f);
+        for (int cidx = ca; cidx < cb; ++cidx) {
+          const float2 h = hn;
+          if (cidx + 1 < cb) hn = hr[cidx + 1];
+          const V hv{h.x, h.y};
+          const V* x = Xs + (size_t)cidx * J;
+#pragma unroll
+          for (int v = 0; v < NV; ++v) v_mac(y[v], hv, x[v]);
+        }
+      }
+      if (it < nloc) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          if (v0 + v >= A.nv) continue;
+          if constexpr (CPLX) Z[((size_t)e * npad + r) * A.nv + v0 + v] = mkc(v_to(v_fin(y[2 * v])), v_to(v_fin(y[2 * v + 1])));
+          else Z[((size_t)e * npad + r) * A.nv + v0 + v] = v_to(v_fin(y[v]));
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < J; ++j) part[(size_t)pidx * J + j] = v_fin(y[j]);
+      }
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < ne * NV; t += NT) {   // enrichment rows: sum of the chunks
+      const int i = t / NV, v = t % NV;
       if (v0 + v >= A.nv) continue;
-      S* z = Z + ((size_t)e * npad + r) * A.nv + v0 + v;
-      const S old = ne > 0 ? *z : S{};
-      if constexpr (CPLX) *z = mkc(old.x + v_to(Ys[(size_t)t * 2]), old.y + v_to(Ys[(size_t)t * 2 + 1]));
-      else *z = old + v_to(Ys[t]);
+      V sr = v_from<V>(0.0), si = v_from<V>(0.0);
+      for (int ch = 0; ch < nch; ++ch) {
+        const V* pp = part + (size_t)(i * nch + ch) * J + v * R;
+        sr = v_add(sr, pp[0]);
+        if (CPLX) si = v_add(si, pp[1]);
+      }
+      if constexpr (CPLX) Z[((size_t)e * npad + nloc + i) * A.nv + v0 + v] = mkc(v_to(sr), v_to(si));
+      else Z[((size_t)e * npad + nloc + i) * A.nv + v0 + v] = v_to(sr);
     }
   }
 }
@@ -188,13 +267,6 @@ int setup_sumfac(oefe_ctx* c) {
   c->d_sf = nullptr;
   c->d_sf_cells = c->d_dense_cells = c->d_sf_index = c->d_dense_index = nullptr;
   c->n_sf = c->n_dense = 0;
-  dev_free(c->d_oz_jobs);
-  dev_free(c->d_oz_jobs_c);
-  c->d_oz_jobs = c->d_oz_jobs_c = nullptr;
-  c->n_oz_jobs = 0;
-  c->sf_cells_h.clear();
-  c->dense_cells_h.clear();
-  c->sf_n1_h.clear();
   const int P = c->P;
   if (P > SF_MAXP || c->nloc != P * P * P) return OEFE_OK;
   std::vector<int> sfc, den;
@@ -203,16 +275,9 @@ int setup_sumfac(oefe_ctx* c) {
   std::vector<double> gx[13], gw[13];
   for (int e = 0; e < c->ncells; ++e) {
     const int l0 = c->leaf_off[e], l1 = c->leaf_off[e + 1];
-    if (l1 - l0 != 1 || c->leaves[l0].n1 > SF_MAXN1) den.push_back(e);
-    else sfc.push_back(e);
-  }
-  // cells with the same rule next to each other: one launch per rule (pair products)
-  std::stable_sort(sfc.begin(), sfc.end(),
-                   [&](int x, int y) { return c->leaves[c->leaf_off[x]].n1 < c->leaves[c->leaf_off[y]].n1; });
-  for (int e : sfc) {
-    const Leaf& L = c->leaves[c->leaf_off[e]];
+    const Leaf& L = c->leaves[l0];
+    if (l1 - l0 != 1 || L.n1 > SF_MAXN1) { den.push_back(e); continue; }
     const int n1 = L.n1;
-    c->sf_n1_h.push_back(n1);
     if (gw[n1].empty()) gauss_rule(n1, gx[n1], gw[n1]);
     n1max = std::max(n1max, n1);
     double lo[3], hi[3];
@@ -249,6 +314,7 @@ int setup_sumfac(oefe_ctx* c) {
           t[SF_A + o] = g1 - g2;
         }
     }
+    sfc.push_back(e);
     tabs.insert(tabs.end(), t.begin(), t.end());
   }
   // work buffers: every intermediate of the contractions (n1 may be below P) and two P^3 blocks
@@ -273,8 +339,6 @@ int setup_sumfac(oefe_ctx* c) {
   OEFE_CUDA_TRY(c, cudaMemcpy(c->d_dense_index, dindex.data(), dindex.size() * sizeof(int), cudaMemcpyHostToDevice));
   c->n_sf = (int)sfc.size();
   c->n_dense = (int)den.size();
-  c->sf_cells_h = sfc;
-  c->dense_cells_h = den;
   return OEFE_OK;
 }
 
@@ -286,8 +350,8 @@ int launch_cell_apply_sf(oefe_ctx* c, const KData& K, const void* X, int ldx, in
   SfArgs A;
   A.sf = c->d_sf;
   A.cells = c->d_sf_cells;
-  A.count = c->n_sf;
   A.H = K.H64;
+  A.Hp = K.Hp;
   A.compact = K.compact ? 1 : 0;
   A.ne_max = c->ne_max;
   A.sf_base = (long long)c->n_dense * c->npad * c->npad;
@@ -311,40 +375,50 @@ int launch_cell_apply_sf(oefe_ctx* c, const KData& K, const void* X, int ldx, in
   auto go = [&](auto kern, size_t smem, int nvb, int nthreads) -> int {
     if (smem > 227 * 1024) { c->err = "sum factorization: work arrays exceed shared memory"; return OEFE_ERR_ARG; }
     OEFE_CUDA_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    dim3 grid((nv + nvb - 1) / nvb, A.count);
+    dim3 grid((nv + nvb - 1) / nvb, c->n_sf);
     OEFE_COUNTED kern<<<grid, nthreads, smem, st>>>(A);
     OEFE_CUDA_TRY(c, cudaGetLastError());
     return OEFE_OK;
   };
   if (c->f64_products == OEFE_F64_PAIRS) {
-    // the blocks with enrichment rows on the tensor cores, then the CFE-CFE block per class of points
-    // per axis (the list is sorted by it): register-tiled instances for the orders and rules in use,
-    // else the general kernel, in the launch shape of oefe_set_product_shape
-    if (!K.pairs) { c->err = "FP32-pair products: build the operator with OEFE_STORE_F64PAIR"; return OEFE_ERR_STATE; }
-    OEFE_TRY(launch_cell_oz(c, K, X, ldx, nv, cplx, Z, st));
-    for (int i = 0; i < c->n_sf;) {
-      const int n1 = c->sf_n1_h[i];
-      int m = i;
-      while (m < c->n_sf && c->sf_n1_h[m] == n1) ++m;
-      bool done = false;
-      OEFE_TRY(launch_sf_cc(c, K, X, ldx, nv, cplx, Z, i, m - i, n1, &done, st));
-      if (!done) {
-        A.sf = c->d_sf + (size_t)i * SF_STRIDE;
-        A.cells = c->d_sf_cells + i;
-        A.count = m - i;
-        const int v = c->sf_variant;
-        int s;
-        if (cplx) s = v == 0 ? go(k_cell_apply_sf<true, 4, f2, 512>, sf_smem<true>(c, 4), 4, 512)
-                    : v == 1 ? go(k_cell_apply_sf<true, 2, f2, 384>, sf_smem<true>(c, 2), 2, 384)
-                             : go(k_cell_apply_sf<true, 2, f2, 512>, sf_smem<true>(c, 2), 2, 512);
-        else s = v == 0 ? go(k_cell_apply_sf<false, 8, f2, 512>, sf_smem<false>(c, 8), 8, 512)
-                 : v == 1 ? go(k_cell_apply_sf<false, 4, f2, 384>, sf_smem<false>(c, 4), 4, 384)
-                          : go(k_cell_apply_sf<false, 4, f2, 512>, sf_smem<false>(c, 4), 4, 512);
-        OEFE_TRY(s);
+    if (!K.Hp) { c->err = "FP32-pair products: build the operator with OEFE_STORE_F64PAIR"; return OEFE_ERR_STATE; }
+    // launch shapes: one CTA of 512 threads per SM over 4 (complex) vectors, or two CTAs of 384 or
+    // of 512 threads per SM over 2 vectors each (half the shared memory, the cell's enrichment
+    // blocks read twice as often); the fastest on this operator is kept after timing each once
+    auto run = [&](int v) -> int {
+      if (cplx) {
+        if (v == 0) return go(k_cell_apply_sf<true, 4, f2, 512>, sf_smem<true>(c, 4), 4, 512);
+        if (v == 1) return go(k_cell_apply_sf<true, 2, f2, 384>, sf_smem<true>(c, 2), 2, 384);
+        return go(k_cell_apply_sf<true, 2, f2, 512>, sf_smem<true>(c, 2), 2, 512);
       }
-      i = m;
+      if (v == 0) return go(k_cell_apply_sf<false, 8, f2, 512>, sf_smem<false>(c, 8), 8, 512);
+      if (v == 1) return go(k_cell_apply_sf<false, 4, f2, 384>, sf_smem<false>(c, 4), 4, 384);
+      return go(k_cell_apply_sf<false, 4, f2, 512>, sf_smem<false>(c, 4), 4, 512);
+    };
+    if (c->sf_variant < 0) {   // first use: time each on this operator (after one warm launch)
+      constexpr int NVAR = 3;
+      cudaEvent_t ev[NVAR + 1];
+      for (auto& e : ev) OEFE_CUDA_TRY(c, cudaEventCreate(&e));
+      int s = run(0);
+      if (s == OEFE_OK) cudaEventRecord(ev[0], st);
+      for (int v = 0; v < NVAR && s == OEFE_OK; ++v) {
+        s = run(v);
+        cudaEventRecord(ev[v + 1], st);
+      }
+      if (s == OEFE_OK) {
+        OEFE_CUDA_TRY(c, cudaEventSynchronize(ev[NVAR]));
+        float best = 1e30f;
+        for (int v = 0; v < NVAR; ++v) {
+          float ms = 0;
+          cudaEventElapsedTime(&ms, ev[v], ev[v + 1]);
+          if (ms < best) { best = ms; c->sf_variant = v; }
+        }
+        // Z holds the last variant's product; the products of all variants are the same numbers
+      }
+      for (auto& e : ev) cudaEventDestroy(e);
+      return s;
     }
-    return OEFE_OK;
+    return run(c->sf_variant);
   }
   if (cplx) return go(k_cell_apply_sf<true, 4, double, SF_THREADS>, sf_smem<true>(c, 4), 4, SF_THREADS);
   return go(k_cell_apply_sf<false, 8, double, SF_THREADS>, sf_smem<false>(c, 8), 8, SF_THREADS);
