@@ -594,7 +594,7 @@ int orthonormalize_t(oefe_ctx* c, int ik, S* X, int nv, int ld, double* cond) {
   const size_t pbytes = (size_t)nchunk * nv * nv * sizeof(S);
   const size_t pbytes_a = ((pbytes + 255) / 256) * 256;
   const size_t dbytes = (((size_t)nv * sizeof(double) + 255) / 256) * 256;
-  OEFE_TRY(ensure_ws(c, wbytes + 3 * sbytes + pbytes_a + dbytes + chol_scratch(nv, sizeof(S))));
+  OEFE_TRY(ensure_ws(c, wbytes + 3 * sbytes + pbytes_a + dbytes + chol_scratch(nv)));
   char* base = (char*)c->ws;
   S* W = (S*)base;
   S* Sm = (S*)(base + wbytes);

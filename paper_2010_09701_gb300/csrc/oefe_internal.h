@@ -254,7 +254,7 @@ int build_hamiltonian(oefe_ctx* c, const double* veff, int store);
 int chol_inverse_inplace(oefe_ctx* c, double* A, int n, bool cplx, bool inverse, int* info_host);
 
 // blocked Cholesky factor and triangular inverse (chol.cu)
-size_t chol_scratch(int n, size_t scalar);
+size_t chol_scratch(int n);
 template <typename S>
 int chol_factor_inverse(oefe_ctx* c, S* A, S* L, S* Y, int n, void* scratch, int* d_info, int* info_host);
 
