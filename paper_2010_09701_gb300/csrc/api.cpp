@@ -80,6 +80,11 @@ int oefe_create(oefe_ctx_t* out, int device, void* cuda_stream) {
     delete c;
     return OEFE_ERR_CUDA;
   }
+  size_t free_bytes = 0;
+  if (cudaMemGetInfo(&free_bytes, &c->dev_bytes) != cudaSuccess) {
+    cudaGetLastError();
+    c->dev_bytes = 0;
+  }
   if (dev_alloc(c, (void**)&c->d_status, 64) != OEFE_OK) {
     delete c;
     return OEFE_ERR_OOM;

@@ -444,6 +444,11 @@ int run_fields(oefe_ctx* c, KData& K, const void* X, int nv, int ld, int dtype, 
   OEFE_TRY(ensure_orth_enrichment(c, K));
   const bool pairs = c->f64_products == OEFE_F64_PAIRS;
   const bool cplx = dtype == OEFE_C128;
+  if (pairs && !X2) {
+    bool done = false;
+    OEFE_TRY(fields_pair(c, K, X, nv, ld, cplx, occ, out, accumulate, scale, out2, &done));
+    if (done) return OEFE_OK;
+  }
   FieldArgs A;
   A.leaves = c->d_leaves;
   A.qxyz = c->d_qxyz;
@@ -523,6 +528,13 @@ int run_fields(oefe_ctx* c, KData& K, const void* X, int nv, int ld, int dtype, 
   return go(k_fields<double, false, 4>, field_smem<double>(c, false, 4, dual));
 }
 
+// end of a fields call: wait, and in pair mode read the tensor-core kernels' error word
+int finish_fields(oefe_ctx* c) {
+  if (c->f64_products == OEFE_F64_PAIRS) return oz_status(c, "fields");
+  OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  return OEFE_OK;
+}
+
 int check_fields(oefe_ctx* c, int ik, const void* X, int nv, int ld, int dtype) {
   if (!c->has_k) { c->err = "call oefe_kpoints first"; return OEFE_ERR_STATE; }
   if (ik < 0 || ik >= (int)c->kd.size()) { c->err = "k index out of range"; return OEFE_ERR_ARG; }
@@ -559,7 +571,8 @@ int density_grad(oefe_ctx* c, int nk, const void* const* X, const int* nv, const
                     ik == ik_grad ? gV : nullptr);
     off += nv[ik];
   }
-  cudaStreamSynchronize(c->stream);
+  if (st == OEFE_OK) st = finish_fields(c);
+  else cudaStreamSynchronize(c->stream);
   dev_free(d_occ);
   return st;
 }
@@ -573,8 +586,7 @@ int band_trace_grad(oefe_ctx* c, int ik, const void* X, int nv, int ld, int dtyp
   OEFE_TRY(check_fields(c, ik, X, nv, ld, dtype));
   if (!gV) { c->err = "need gV"; return OEFE_ERR_ARG; }
   OEFE_TRY(run_fields(c, c->kd[ik], X, nv, ld, dtype, nullptr, gV, false));
-  OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  return OEFE_OK;
+  return finish_fields(c);
 }
 
 // d/dV_q of Re sum conj(G) (H X) = w_q Re sum_v conj(u_G,v(x_q)) u_X,v(x_q), one fields pass over the
@@ -585,6 +597,5 @@ int fields_cross(oefe_ctx* c, int ik, const void* X, const void* G, int nv, int 
   if (!gV) { c->err = "need gV"; return OEFE_ERR_ARG; }
   if (G) OEFE_TRY(run_fields(c, c->kd[ik], X, nv, ld, dtype, nullptr, gV, false, scale, G, ld));
   else OEFE_TRY(run_fields(c, c->kd[ik], X, nv, ld, dtype, nullptr, gV, false, scale));
-  OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  return OEFE_OK;
+  return finish_fields(c);
 }

@@ -106,6 +106,7 @@ struct oefe_ctx {
   cudaStream_t stream = nullptr;
   std::string err;
   int num_sms = 0;
+  size_t dev_bytes = 0;   // the device's memory
 
   // mesh
   bool has_mesh = false;
@@ -322,6 +323,11 @@ int density(oefe_ctx* c, int nk, const void* const* X, const int* nv, const int*
 int density_grad(oefe_ctx* c, int nk, const void* const* X, const int* nv, const int* ld, int dtype, const double* occ,
                  double* rho, int ik_grad, double* gV);
 int band_trace_grad(oefe_ctx* c, int ik, const void* X, int nv, int ld, int dtype, double* gV);
+// the same sums in pair mode, enrichment part on the tensor cores (fields_pair.cu)
+int fields_pair(oefe_ctx* c, KData& K, const void* X, int nv, int ld, bool cplx, const double* occ, double* out,
+                bool density, double scale, double* out2, bool* done);
+// reads and clears the tensor-core kernels' error word (after a stream synchronization it joins)
+int oz_status(oefe_ctx* c, const char* what);
 // adjoint.cu
 int band_trace(oefe_ctx* c, int ik, const void* X, int nv, int ld, int dtype, double* e, void* HX);
 int band_trace_vjp(oefe_ctx* c, int ik, const void* X, int nv, int ld, int dtype, double alpha, double* gV, void* gX);

@@ -77,6 +77,51 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b
       : "memory");
 }
 
+// The same two issued by a whole warp in step, of which the elected lane (lead = 1, from elect_lane)
+// performs the operation: the warp's control flow stays uniform, so descriptors live in uniform
+// registers and advance by uniform adds. Issued from a one-thread branch, every MMA first moves its
+// operands from vector to uniform registers, about 170 clocks an MMA whatever its shape.
+__device__ __forceinline__ uint32_t elect_lane() {
+  uint32_t lead;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(lead)::"memory");
+  return lead;
+}
+__device__ __forceinline__ void mma_bf16_lead(uint32_t lead, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
+                                              uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(lead)
+      : "memory");
+}
+__device__ __forceinline__ void mma_commit_lead(uint32_t lead, uint64_t* bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_u32(bar)),
+      "r"(lead)
+      : "memory");
+}
+
+// The digit products of levels d = s + t < S into accumulators d (NCOL tensor-memory columns apart):
+// A planes PA bytes apart at shared address a0, B planes PB bytes apart at b0, nks <= KS steps of 16
+// entries; the first product of a level overwrites its accumulator when `fresh`. By a whole warp (see
+// elect_lane), unrolled on two descriptors and constant offsets.
+template <int S, int KS, int PA, int PB, int NCOL>
+__device__ __forceinline__ void issue_digit_levels(uint32_t lead, uint32_t taddr, uint32_t a0, uint32_t b0, uint32_t idesc, int nks,
+                                                   bool fresh) {
+  const uint64_t da = sdesc(a0), db = sdesc(b0);
+#pragma unroll
+  for (int ks = 0; ks < KS; ++ks)
+    if (ks < nks) {
+#pragma unroll
+      for (int s = 0; s < S; ++s)
+#pragma unroll
+        for (int t = 0; t + s < S; ++t)
+          mma_bf16_lead(lead, taddr + (s + t) * NCOL, da + (uint64_t)((s * PA + ks * 32) >> 4), db + (uint64_t)((t * PB + ks * 32) >> 4),
+                   idesc, (s == 0 && ks == 0 && fresh) ? 0u : 1u);
+    }
+}
+
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
