@@ -39,9 +39,6 @@ static void free_all(oefe_ctx* c) {
   dev_free(c->d_dense_cells);
   dev_free(c->d_sf_index);
   dev_free(c->d_dense_index);
-  dev_free(c->d_rotp);
-  c->d_rotp = nullptr;
-  c->rotp_bytes = 0;
   dev_free(c->d_ozpart);
   c->d_ozpart = nullptr;
   c->ozpart_bytes = 0;
@@ -392,12 +389,9 @@ int oefe_release_workspace(oefe_ctx_t ctx) {
   dev_free(ctx->ws2);
   ctx->ws = ctx->ws2 = nullptr;
   ctx->ws_bytes = ctx->ws2_bytes = 0;
-  dev_free(ctx->d_ozpart);   // digit planes of the tensor-core Gram matrices and rotations
+  dev_free(ctx->d_ozpart);   // digit planes and partial sums of the tensor-core Gram matrices and rotations
   ctx->d_ozpart = nullptr;
   ctx->ozpart_bytes = 0;
-  dev_free(ctx->d_rotp);
-  ctx->d_rotp = nullptr;
-  ctx->rotp_bytes = 0;
   return OEFE_OK;
 }
 

@@ -174,8 +174,6 @@ struct oefe_ctx {
   size_t ws_bytes = 0;
   void* ws2 = nullptr;
   size_t ws2_bytes = 0;
-  void* d_rotp = nullptr;               // the small matrix of a pair rotation, as pairs
-  size_t rotp_bytes = 0;
   void* d_ozpart = nullptr;             // partial sums of the tensor-core Gram matrices
   size_t ozpart_bytes = 0;
   int* d_status = nullptr;        // device status word (Cholesky failures, timeouts)
@@ -247,8 +245,11 @@ int rotate_ozaki(oefe_ctx* c, S* X, int ldx, int64_t n, int nv, const S* C, bool
 // the same for any nv, the digits cut inside the MMA kernels (ozaki_wide.cu)
 template <typename S>
 int gram_ozaki_wide(oefe_ctx* c, const S* X, int ldx, const S* W, int ldw, int64_t n, int nv, S* out, bool herm);
+// Gram matrices and rotations of wider blocks from eight digits (oz8_wide.cu)
 template <typename S>
-int rotate_ozaki_wide(oefe_ctx* c, S* X, int ldx, int64_t n, int nv, const S* C, bool herm);
+int gram_oz8(oefe_ctx* c, const S* X, int ldx, const S* W, int ldw, int64_t n, int nv, S* out, bool herm);
+template <typename S>
+int rotate_oz8(oefe_ctx* c, S* X, int ldx, int64_t n, int nv, const S* C, bool herm);
 int build_hamiltonian(oefe_ctx* c, const double* veff, int store);
 
 // dense helpers (linalg.cu)

@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(OZ_T, 1) k_gram_oz(const OzArgs A) {
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5;
+  const bool warp0 = __shfl_sync(0xffffffffu, warp, 0) == 0;   // (uniform)
   const int half = blockIdx.y;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
@@ -200,19 +201,11 @@ __global__ void __launch_bounds__(OZ_T, 1) k_gram_oz(const OzArgs A) {
     const int E = A.ea[p * 128 + row];
     if (tid < OZ_N) Fexp[tid] = A.eb[p * 128 + half * OZ_N + tid];
     // ---- the digit products of levels d = s + t <= 6 into accumulator d
-    if (tid == 0) {
+    if (warp0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll 1
-      for (int d = 0; d < OZ_S; ++d)
-#pragma unroll 1
-        for (int s = 0; s <= d; ++s) {
-          const int t = d - s;
-#pragma unroll
-          for (int ks = 0; ks < OZ_K / 16; ++ks)
-            mma_bf16(taddr + d * OZ_N, sdesc(smem_u32(sA + s * PL) + ks * 32), sdesc(smem_u32(sB + t * BH) + ks * 32),
-                     ID, (s == 0 && ks == 0) ? 0u : 1u);
-        }
-      mma_commit(&mma_bar);
+      const uint32_t lead = elect_lane();
+      issue_digit_levels<OZ_S, OZ_K / 16, PL, BH, OZ_N>(lead, taddr, smem_u32(sA), smem_u32(sB), ID, OZ_K / 16, true);
+      mma_commit_lead(lead, &mma_bar);
     }
     mma_out = true;
     ok = mbar_wait(&mma_bar, (uint32_t)(it & 1), &s_fail);
@@ -419,6 +412,7 @@ __global__ void __launch_bounds__(OZ_T, 1) k_rot_oz(const RotArgs A) {
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5;
+  const bool warp0 = __shfl_sync(0xffffffffu, warp, 0) == 0;   // (uniform)
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                  "r"(OZ_TCOLS)
@@ -456,19 +450,11 @@ __global__ void __launch_bounds__(OZ_T, 1) k_rot_oz(const RotArgs A) {
     bool ok = mbar_wait(&ld_bar, (uint32_t)(it & 1), &s_fail);
     if (__syncthreads_or(!ok)) { s_fail = 1; break; }
     loads_out = false;
-    if (tid == 0) {
+    if (warp0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll 1
-      for (int d = 0; d < OZ_S; ++d)
-#pragma unroll 1
-        for (int s = 0; s <= d; ++s) {
-          const int t = d - s;
-#pragma unroll
-          for (int ks = 0; ks < OZ_K / 16; ++ks)
-            mma_bf16(taddr + d * OZ_N, sdesc(smem_u32(sA + s * PL) + ks * 32), sdesc(smem_u32(sB + t * BH) + ks * 32),
-                     ID, (kh == 0 && s == 0 && ks == 0) ? 0u : 1u);
-        }
-      mma_commit(&mma_bar);
+      const uint32_t lead = elect_lane();
+      issue_digit_levels<OZ_S, OZ_K / 16, PL, BH, OZ_N>(lead, taddr, smem_u32(sA), smem_u32(sB), ID, OZ_K / 16, kh == 0);
+      mma_commit_lead(lead, &mma_bar);
     }
     mma_out = true;
     ok = mbar_wait(&mma_bar, (uint32_t)(it & 1), &s_fail);

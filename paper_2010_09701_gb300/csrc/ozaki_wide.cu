@@ -1,26 +1,19 @@
-// FP64-class Gram matrices and rotations of wide vector blocks (more than the 64 vectors the
-// plane-based kernels of ozaki_gram.cu take) on the tensor cores, with the same exact bf16 digit
+// FP64-class Gram matrices of wide vector blocks (more than the 64 vectors the plane-based kernels of
+// ozaki_gram.cu take) on the tensor cores, for the projected matrices of Rayleigh-Ritz (the signs of its
+// vectors follow their last bits; oz8_wide.cu is the faster kernel), with the same exact bf16 digit
 // slicing (the Ozaki scheme): every operand value is cut into 7 digits of 7 bits under a common
 // exponent per operand row and K chunk, the 28 digit products of levels d = s + t <= 6 are
 // accumulated exactly in FP32 in tensor memory (7 accumulators of 64 columns), and the levels are
 // combined in FP32 pairs, scaled by exact powers of two and summed over the chunks in pairs.
 //
 // Unlike the plane-based kernels, the digits are cut inside the MMA kernels into shared memory
-// (nothing is staged in global memory but the small rotation matrix's digits), so wide blocks need
-// no digit planes the size of the operands. One round = one K chunk of 64 real entries for one
+// (nothing is staged in global memory), so wide blocks need no digit planes the size of the operands. One round = one K chunk of 64 real entries for one
 // tile of 128 operand rows and 64 output columns: 112 MMAs (M 128, N 64, K 16).
 //
 //   Gram S = X^+ W: real form A = [Re X | Im X]^T (2 nv operand rows, nv for real data), B = [Re W |
 //   Im W] (2 nv columns); K = the rows of the blocks in passes of 64. A CTA takes one (128-row,
 //   64-column) tile of D = A B over a range of passes; D's partial sums are combined afterwards:
 //   Re S = D[i][j] + D[nv+i][nv+j], Im S = D[i][nv+j] - D[nv+i][j].
-//
-//   Rotation X <- X G: A = rows of X, a K chunk = 64 columns (real) or [Re | Im] of 32 complex
-//   columns; B = the matching rows of the real form of G for 64 output columns (the real parts, or
-//   the imaginary parts, of 64 complex output columns). A CTA takes whole tiles of 128 rows, the K
-//   chunks outermost (the A digits of a chunk cut once for all output blocks), every output block's
-//   FP32-pair partial sums in a staging area, so the in-place update never reads a row it has
-//   written.
 //
 // Every wait is bounded; on a timeout the CTA raises the error flag, lets its copies and MMAs in
 // flight land, frees its tensor memory and returns.
@@ -58,21 +51,6 @@ __device__ __forceinline__ void put_pair(unsigned char* base, int plane_bytes, i
 #pragma unroll
   for (int s = 0; s < OZ_S; ++s)
     *reinterpret_cast<__nv_bfloat162*>(base + (size_t)s * plane_bytes + swz(r, kk)) = __floats2bfloat162_rn(c0[s], c1[s]);
-}
-
-// thread 0: the digit products of levels d = s + t <= 6 into accumulator d
-__device__ __forceinline__ void issue_round(uint32_t taddr, uint32_t sA, uint32_t sB) {
-  constexpr uint32_t ID = idesc_bf16(128, WN, false);
-#pragma unroll 1
-  for (int d = 0; d < OZ_S; ++d)
-#pragma unroll 1
-    for (int s = 0; s <= d; ++s) {
-      const int t = d - s;
-#pragma unroll
-      for (int ks = 0; ks < WK / 16; ++ks)
-        mma_bf16(taddr + d * WN, sdesc(sA + s * PLA + ks * 32), sdesc(sB + t * PLB + ks * 32), ID,
-                 (s == 0 && ks == 0) ? 0u : 1u);
-    }
 }
 
 // the levels of (row, 32 columns ch*32 ..) combined and added to the running pair sums R:
@@ -166,6 +144,7 @@ __global__ void __launch_bounds__(WT, 1) k_gram_wide(const WGramArgs A) {
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5;
+  const bool warp0 = __shfl_sync(0xffffffffu, warp, 0) == 0;   // (uniform)
   if (warp == 0) tmem_alloc_cta(&tmem_slot);
   if (tid == 0) {
     mbar_init(&mma_bar, 1);
@@ -226,10 +205,11 @@ __global__ void __launch_bounds__(WT, 1) k_gram_wide(const WGramArgs A) {
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
-    if (tid == 0) {
+    if (warp0) {   // the digit products of levels d = s + t <= 6 into accumulator d
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      issue_round(taddr, smem_u32(sA), smem_u32(sB));
-      mma_commit(&mma_bar);
+      const uint32_t lead = elect_lane();
+      issue_digit_levels<OZ_S, WK / 16, PLA, PLB, WN>(lead, taddr, smem_u32(sA), smem_u32(sB), idesc_bf16(128, WN, false), WK / 16, true);
+      mma_commit_lead(lead, &mma_bar);
     }
     mma_out = true;
     const bool ok = mbar_wait(&mma_bar, (uint32_t)(it & 1), &s_fail);
@@ -268,206 +248,6 @@ __global__ void k_gram_wide_reduce(const double* part, int nbx, int nI, int nJ, 
   };
   if constexpr (sizeof(S) == sizeof(cd)) out[t] = mkc(D(i, j) + D(nv + i, nv + j), D(i, nv + j) - D(nv + i, j));
   else out[t] = D(i, j);
-}
-
-// ------------------------------------------------------------------ rotation X <- X G
-// A K entry kk of chunk kc: real data column kc * 64 + kk; complex data [Re | Im] of the columns
-// kc * 32 + (kk mod 32)
-__device__ __forceinline__ double rot_op(const void* X, int ldx, long long g, int kc, int kk, int nv, bool cplx) {
-  if (!cplx) {
-    const int j = kc * 64 + kk;
-    return j < nv ? reinterpret_cast<const double*>(X)[g * ldx + j] : 0.0;
-  }
-  const int j = kc * 32 + (kk & 31);
-  if (j >= nv) return 0.0;
-  const cd v = reinterpret_cast<const cd*>(X)[g * ldx + j];
-  return kk < 32 ? v.x : v.y;
-}
-
-// digits of the real form of G for every (K chunk, output block), one thread per output column:
-// planes [(kc, ob)][digit][64 columns][64 k], exponents [(kc, ob)][64]. G[k][j] = herm ?
-// (k <= j ? conj(C[j][k]) : 0) : C[k][j]. Output block ob: real data columns ob * 64 ..; complex
-// data the real (nh = 0) or imaginary (nh = 1) parts of columns (ob / 2) * 64 ..
-template <typename S>
-__global__ void k_rot_wide_bdigits(const S* C, int nv, bool herm, int nkc, int nob, unsigned char* planes, int* exps) {
-  constexpr bool CPLX = sizeof(S) == sizeof(cd);
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= (long long)nkc * nob * WN) return;
-  const int n = (int)(t % WN), ob = (int)((t / WN) % nob), kc = (int)(t / ((long long)WN * nob));
-  auto G = [&](int k, int j) -> cd {
-    if (k >= nv || j >= nv) return mkc(0, 0);
-    if (herm) {
-      if (k > j) return mkc(0, 0);
-      if constexpr (CPLX) return cconj(C[(size_t)j * nv + k]);
-      else return mkc(C[(size_t)j * nv + k], 0.0);
-    }
-    if constexpr (CPLX) return C[(size_t)k * nv + j];
-    else return mkc(C[(size_t)k * nv + j], 0.0);
-  };
-  auto Bv = [&](int kk) -> double {
-    if (!CPLX) return G(kc * 64 + kk, ob * WN + n).x;
-    const int nh = ob & 1, col = (ob >> 1) * WN + n;
-    const cd g = G(kc * 32 + (kk & 31), col);
-    if (kk < 32) return nh == 0 ? g.x : g.y;   // Re X rows
-    return nh == 0 ? -g.y : g.x;              // Im X rows
-  };
-  int mex = 0;
-  for (int kk = 0; kk < WK; ++kk) mex = max(mex, bexp(Bv(kk)));
-  const int E = mex ? mex - 1022 : 0;
-  const size_t blk = (size_t)kc * nob + ob;
-  exps[blk * WN + n] = E;
-  for (int kp = 0; kp < WK / 2; ++kp)
-    put_pair(planes + blk * OZ_S * PLB, PLB, n, 2 * kp, Bv(2 * kp), Bv(2 * kp + 1), E);
-}
-
-struct WRotArgs {
-  void* X;
-  int ldx;
-  long long n;
-  int nv;
-  bool cplx;
-  int nkc, nob;
-  bool herm;                 // G upper triangular: K chunks past an output block's columns are zero
-  const unsigned char* bpl;  // B digit planes per (kc, ob)
-  const int* bex;            // B exponents per (kc, ob)
-  float2* stage;             // per CTA: [ob][128 rows][64 columns] FP32-pair partial sums
-  int* err;
-};
-
-// K chunk kc contributes to output block ob (an upper triangular G has no entries in the chunks past
-// the block's last column)
-__device__ __forceinline__ bool rot_active(const WRotArgs& A, int kc, int ob) {
-  return !A.herm || kc < (A.cplx ? 2 * (ob >> 1) + 2 : ob + 1);
-}
-
-// Per tile of 128 rows the K chunks run outermost: the A digits of a chunk are cut once (a warp per
-// 16 rows, a lane per pair of K entries: coalesced loads, a row's exponent by one warp reduction)
-// and serve every output block the chunk contributes to; each (chunk, block) round's combined
-// levels are added to the block's FP32-pair partial sums staged per CTA (the first chunk stores),
-// and the tile's rows of X are rewritten from the stage once every chunk is done.
-__global__ void __launch_bounds__(WT, 1) k_rot_wide(const WRotArgs A) {
-  extern __shared__ __align__(1024) unsigned char wz_raw[];
-  unsigned char* sm = (unsigned char*)(((uintptr_t)wz_raw + 1023) & ~(uintptr_t)1023);
-  unsigned char* sA = sm;
-  unsigned char* sB = sm + OZ_S * PLA;
-  __shared__ int sE[128], Fexp[WN];
-  __shared__ uint64_t b_bar, mma_bar;
-  __shared__ uint32_t tmem_slot;
-  __shared__ volatile int s_fail;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (warp == 0) tmem_alloc_cta(&tmem_slot);
-  if (tid == 0) {
-    mbar_init(&b_bar, 1);
-    mbar_init(&mma_bar, 1);
-    s_fail = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t taddr = tmem_slot;
-  const int row = tid & 127, ch = tid >> 7;
-  const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
-  float2* stage = A.stage + (size_t)blockIdx.x * A.nob * 128 * WN;
-  double* Xd = reinterpret_cast<double*>(A.X);
-  const long long ldr = (long long)A.ldx * (A.cplx ? 2 : 1);
-  const long long tiles = (A.n + 127) / 128;
-  long long it = 0;   // rounds so far: the phase of both barriers
-  bool b_out = false, mma_out = false;
-  for (long long tile = blockIdx.x; tile < tiles && !s_fail; tile += gridDim.x) {
-    const long long r0 = tile * 128;
-    const int nr = (int)min(128ll, A.n - r0);
-    for (int kc = 0; kc < A.nkc && !s_fail; ++kc) {
-      {   // A digits of the chunk: warp w takes rows 16 w .. 16 w + 15, lane l the K entries 2 l, 2 l + 1
-        double v[32];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int r = warp * 16 + i;
-          const bool ok = r < nr;
-          v[2 * i] = ok ? rot_op(A.X, A.ldx, r0 + r, kc, 2 * lane, A.nv, A.cplx) : 0.0;
-          v[2 * i + 1] = ok ? rot_op(A.X, A.ldx, r0 + r, kc, 2 * lane + 1, A.nv, A.cplx) : 0.0;
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int r = warp * 16 + i;
-          const int mex = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(bexp(v[2 * i]), bexp(v[2 * i + 1])));
-          const int E = mex ? mex - 1022 : 0;
-          if (lane == 0) sE[r] = E;
-          put_pair(sA, PLA, r, 2 * lane, v[2 * i], v[2 * i + 1], E);
-        }
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      __syncthreads();
-      for (int ob = 0; ob < A.nob; ++ob, ++it) {
-        if (!rot_active(A, kc, ob)) { --it; continue; }
-        const size_t blk = (size_t)kc * A.nob + ob;
-        if (tid < WN) Fexp[tid] = A.bex[blk * WN + tid];
-        if (tid == 0) {   // the round's B digits, then its 112 MMAs
-          mbar_expect_tx(&b_bar, (uint32_t)(OZ_S * PLB));
-          bulk_copy(smem_u32(sB), A.bpl + blk * OZ_S * PLB, (uint32_t)(OZ_S * PLB), &b_bar);
-          b_out = true;
-          if (mbar_wait(&b_bar, (uint32_t)(it & 1), &s_fail)) {
-            b_out = false;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            issue_round(taddr, smem_u32(sA), smem_u32(sB));
-            mma_commit(&mma_bar);
-          } else {
-            s_fail = 1;
-          }
-        }
-        __syncthreads();
-        if (s_fail) break;
-        mma_out = true;
-        const bool ok = mbar_wait(&mma_bar, (uint32_t)(it & 1), &s_fail);
-        if (__syncthreads_or(!ok)) { s_fail = 1; break; }
-        mma_out = false;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        f2 R[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) R[j] = f2{0.0f, 0.0f};
-        add_levels(taddr, lane_base, ch, sE[row], Fexp, R);
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        // the block's partial sums of (row, 32 columns ch 32 ..): 256 contiguous bytes per thread
-        float4* st = reinterpret_cast<float4*>(stage + ((size_t)ob * 128 + row) * WN + ch * 32);
-        if (kc == 0) {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) st[j] = make_float4(R[2 * j].h, R[2 * j].l, R[2 * j + 1].h, R[2 * j + 1].l);
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const float4 o = st[j];
-            const f2 a = f2_add(f2{o.x, o.y}, R[2 * j]), b = f2_add(f2{o.z, o.w}, R[2 * j + 1]);
-            st[j] = make_float4(a.h, a.l, b.h, b.l);
-          }
-        }
-        __syncthreads();
-      }
-    }
-    if (s_fail) break;
-    // every chunk of the tile is done: its rows of X from the stage (a thread per real of a row)
-    for (int ob = 0; ob < A.nob; ++ob)
-      for (int t = tid; t < nr * WN; t += WT) {
-        const int r = t / WN, col = t % WN;
-        const float2 v = stage[((size_t)ob * 128 + r) * WN + col];
-        const double x = f2_to(f2{v.x, v.y});
-        if (!A.cplx) {
-          const int c = ob * WN + col;
-          if (c < A.nv) Xd[(r0 + r) * ldr + c] = x;
-        } else {
-          const int c = (ob >> 1) * WN + col;
-          if (c < A.nv) Xd[(r0 + r) * ldr + 2 * c + (ob & 1)] = x;
-        }
-      }
-    __syncthreads();
-  }
-  if (tid == 0 && s_fail) {
-    if (mma_out) mbar_wait_drain(&mma_bar, (uint32_t)(it & 1));
-    if (b_out) mbar_wait_drain(&b_bar, (uint32_t)(it & 1));
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (s_fail && tid == 0) atomicExch(A.err, 1);
-  if (warp == 0) tmem_free_cta(taddr);
 }
 
 int grow_ozpart(oefe_ctx* c, size_t need) {
@@ -536,41 +316,5 @@ int gram_ozaki_wide(oefe_ctx* c, const S* X, int ldx, const S* W, int ldw, int64
   return finish_wide(c, "gram");
 }
 
-// X[0:n] <- X G (G = C, or C^+ of a lower triangular C when herm) on the tensor cores, any nv
-template <typename S>
-int rotate_ozaki_wide(oefe_ctx* c, S* X, int ldx, int64_t n, int nv, const S* C, bool herm) {
-  constexpr bool CPLX = sizeof(S) == sizeof(cd);
-  const int nkc = CPLX ? (nv + 31) / 32 : (nv + 63) / 64;
-  const int nob = CPLX ? 2 * ((nv + WN - 1) / WN) : (nv + WN - 1) / WN;
-  const long long tiles = (n + 127) / 128;
-  const int grid = (int)std::max<long long>(1, std::min<long long>(tiles, c->num_sms));
-  auto a256 = [](size_t x) { return ((x + 255) / 256) * 256; };
-  const size_t pl_bytes = a256((size_t)nkc * nob * OZ_S * PLB), ex_bytes = a256((size_t)nkc * nob * WN * sizeof(int));
-  const size_t st_bytes = a256((size_t)grid * nob * 128 * WN * sizeof(float2));
-  OEFE_TRY(grow_ozpart(c, pl_bytes + ex_bytes + st_bytes));
-  unsigned char* base = (unsigned char*)c->d_ozpart;
-  WRotArgs A;
-  A.X = X;
-  A.ldx = ldx;
-  A.n = n;
-  A.nv = nv;
-  A.cplx = CPLX;
-  A.nkc = nkc;
-  A.nob = nob;
-  A.herm = herm;
-  A.bpl = base;
-  A.bex = (const int*)(base + pl_bytes);
-  A.stage = (float2*)(base + pl_bytes + ex_bytes);
-  A.err = c->d_status + 2;
-  const long long nb = (long long)nkc * nob * WN;
-  OEFE_COUNTED k_rot_wide_bdigits<S><<<(unsigned)((nb + 127) / 128), 128, 0, c->stream>>>(C, nv, herm, nkc, nob, base,
-                                                                                           (int*)(base + pl_bytes));
-  OEFE_CUDA_TRY(c, cudaFuncSetAttribute(k_rot_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WSMEM));
-  OEFE_COUNTED k_rot_wide<<<grid, WT, WSMEM, c->stream>>>(A);
-  return finish_wide(c, "rotate");
-}
-
 template int gram_ozaki_wide<double>(oefe_ctx*, const double*, int, const double*, int, int64_t, int, double*, bool);
 template int gram_ozaki_wide<cd>(oefe_ctx*, const cd*, int, const cd*, int, int64_t, int, cd*, bool);
-template int rotate_ozaki_wide<double>(oefe_ctx*, double*, int, int64_t, int, const double*, bool);
-template int rotate_ozaki_wide<cd>(oefe_ctx*, cd*, int, int64_t, int, const cd*, bool);
