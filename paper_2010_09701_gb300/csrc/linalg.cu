@@ -209,20 +209,60 @@ __global__ void k_rotate(S* X, int ldx, int64_t n, int nv, const S* C, bool herm
   }
 }
 
-// Column norms for residuals: out[v] = sum_rows conj(R) M^{-1} R, with the
-// lumped block divided by m and the enrichment block through (M^oo)^{-1}.
+// Residual norms of the rotated block, numerators ||H u - eps M u||^2_{M^-1} per column: partial sums over
+// the lumped rows from H U and U (M u is a product with the mass, not a third rotated block), one CTA
+// per range of rows, a thread per column. Bound: the two blocks' bytes and three FP64 operations an
+// entry; the divisions by the mass are one per row (per entry they took 7.4 ms at 885 k x 360).
+constexpr int RN_T = 256, RN_R = 64;
 template <typename S>
-__global__ void k_resid_norms(const S* R, int ldr, const double* m, const S* Mooinv, int64_t nh, int nO, int nv,
-                              double* out) {
-  const int v = blockIdx.x;
-  double s = 0.0;
-  for (int64_t r = threadIdx.x; r < nh; r += blockDim.x) {
-    const S x = R[r * ldr + v];
-    s += Ops<S>::re(Ops<S>::mulc(x, x)) / m[r];
+__global__ void __launch_bounds__(RN_T) k_resid_partial(const S* HU, int ldh, const S* U, int ldu, const double* m,
+                                                        const double* eps, int64_t nh, int nv, int64_t rows, double* part) {
+  __shared__ double ms[RN_R], mi[RN_R];
+  const int64_t r0 = blockIdx.x * rows, r1 = min(nh, r0 + rows);
+  for (int v0 = 0; v0 < nv; v0 += RN_T) {
+    const int v = v0 + threadIdx.x;
+    const double ev = v < nv ? eps[v] : 0.0;
+    double s = 0.0;
+    for (int64_t rb = r0; rb < r1; rb += RN_R) {
+      const int nr = (int)min((int64_t)RN_R, r1 - rb);
+      __syncthreads();
+      if ((int)threadIdx.x < nr) {
+        ms[threadIdx.x] = m[rb + threadIdx.x];
+        mi[threadIdx.x] = 1.0 / ms[threadIdx.x];
+      }
+      __syncthreads();
+      if (v < nv) {
+#pragma unroll 4
+        for (int i = 0; i < nr; ++i) {
+          const S r = HU[(rb + i) * ldh + v] - Ops<S>::scale(U[(rb + i) * ldu + v], ev * ms[i]);
+          s = fma(Ops<S>::re(Ops<S>::mulc(r, r)), mi[i], s);
+        }
+      }
+    }
+    if (v < nv) part[(size_t)blockIdx.x * nv + v] = s;
   }
-  for (int t = threadIdx.x; t < nO * nO; t += blockDim.x) {
+}
+
+// the sums of the partials plus the enrichment rows through (M^oo)^{-1}: a CTA per column
+template <typename S>
+__global__ void __launch_bounds__(256) k_resid_final(const S* HU, int ldh, const S* U, int ldu, const S* Moo, const S* Mooinv,
+                                                     const double* eps, const double* part, int nparts, int64_t nh, int nO,
+                                                     int nv, double* out) {
+  extern __shared__ double rf_raw[];
+  S* r = reinterpret_cast<S*>(rf_raw);   // nO
+  const int v = blockIdx.x;
+  const double ev = eps[v];
+  for (int i = threadIdx.x; i < nO; i += 256) {
+    S w = Ops<S>::zero();
+    for (int j = 0; j < nO; ++j) w = fma_n(Moo[(size_t)i * nO + j], U[(nh + j) * ldu + v], w);
+    r[i] = HU[(nh + i) * ldh + v] - Ops<S>::scale(w, ev);
+  }
+  __syncthreads();
+  double s = 0.0;
+  for (int b = threadIdx.x; b < nparts; b += 256) s += part[(size_t)b * nv + v];
+  for (int t = threadIdx.x; t < nO * nO; t += 256) {
     const int i = t / nO, j = t % nO;
-    s += Ops<S>::re(Ops<S>::mulc(R[(nh + i) * ldr + v], Ops<S>::mul(Mooinv[t], R[(nh + j) * ldr + v])));
+    s += Ops<S>::re(Ops<S>::mulc(r[i], Ops<S>::mul(Mooinv[t], r[j])));
   }
   __shared__ double red[256];
   red[threadIdx.x] = s;
@@ -289,17 +329,6 @@ __global__ void k_scale_cols(S* X, int ldx, int64_t n, int nv, const double* d) 
     const int64_t r = t / nv;
     const int v = (int)(t % nv);
     X[r * ldx + v] = Ops<S>::scale(X[r * ldx + v], d[v]);
-  }
-}
-
-// R = HX - MX diag(eps)
-template <typename S>
-__global__ void k_resid_vec(const S* HX, const S* MX, int ld, const double* eps, int64_t n, int nv, S* R) {
-  const int64_t total = n * nv;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int v = (int)(t % nv);
-    const int64_t r = t / nv;
-    R[r * ld + v] = HX[r * ld + v] - Ops<S>::scale(MX[r * ld + v], eps[v]);
   }
 }
 
@@ -525,12 +554,16 @@ int rayleigh_ritz_t(oefe_ctx* c, int ik, S* X, int nv, int ld, int dtype, double
   OEFE_TRY(rotate<S>(c, X, ld, n, nv, U, false));
   if (resid) {
     OEFE_TRY(rotate<S>(c, HX, nv, n, nv, U, false));
-    OEFE_TRY(rotate<S>(c, MX, nv, n, nv, U, false));
-    const int64_t tot = n * nv;
-    const int blocks = (int)std::min<int64_t>((tot + 255) / 256, (int64_t)c->num_sms * 32);
-    OEFE_COUNTED k_resid_vec<S><<<blocks, 256, 0, c->stream>>>(HX, MX, nv, d_eps, n, nv, HX);  // HX <- residual
     double* d_num = d_eps + nv;
-    OEFE_COUNTED k_resid_norms<S><<<nv, 256, 0, c->stream>>>(HX, nv, c->d_m, (const S*)K.Mooinv, c->nh, c->nO, nv, d_num);
+    const int nparts = std::min(2 * c->num_sms, (int)((c->nh + RN_R - 1) / RN_R));
+    const int64_t rows = (c->nh + nparts - 1) / nparts;
+    double* rp = (double*)MX;   // M X is in the Gram matrix already
+    OEFE_COUNTED k_resid_partial<S><<<nparts, RN_T, 0, c->stream>>>(HX, nv, X, ld, c->d_m, d_eps, c->nh, nv, rows, rp);
+    const size_t rsm = (size_t)std::max(c->nO, 1) * sizeof(S);
+    OEFE_CUDA_TRY(c, cudaFuncSetAttribute(k_resid_final<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm));
+    OEFE_COUNTED k_resid_final<S><<<nv, 256, rsm, c->stream>>>(HX, nv, X, ld, (const S*)K.Moo, (const S*)K.Mooinv, d_eps, rp, nparts,
+                                                               c->nh, c->nO, nv, d_num);
+    OEFE_CUDA_TRY(c, cudaGetLastError());
     // ||u_v||_M^2 = (U^+ (X^+ M X) U)[v][v] from the Gram matrix taken before the rotation
     double* d_den = d_num + nv;
     OEFE_COUNTED k_quad_diag<S><<<nv, 256, 0, c->stream>>>(Mq, U, nv, d_den);
