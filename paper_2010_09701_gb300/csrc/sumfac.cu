@@ -420,8 +420,11 @@ int launch_cell_apply_sf(oefe_ctx* c, const KData& K, const void* X, int ldx, in
     }
     return run(c->sf_variant);
   }
-  if (cplx) return go(k_cell_apply_sf<true, 4, double, SF_THREADS>, sf_smem<true>(c, 4), 4, SF_THREADS);
-  return go(k_cell_apply_sf<false, 8, double, SF_THREADS>, sf_smem<false>(c, 8), 8, SF_THREADS);
+  // 4 real columns per CTA: two CTAs and more per SM, so that one's gather, tables and barriers run under
+  // another's FP64 work (with 8 columns one CTA filled the SM's shared memory at p = 6: 12.4 ms for 64
+  // complex columns of the 8-atom cell, 11.1 with 4)
+  if (cplx) return go(k_cell_apply_sf<true, 2, double, SF_THREADS>, sf_smem<true>(c, 2), 2, SF_THREADS);
+  return go(k_cell_apply_sf<false, 4, double, SF_THREADS>, sf_smem<false>(c, 4), 4, SF_THREADS);
 }
 
 // FP64 operations (an FMA counts two) of one FP64 application of the cell products to nv vectors:
