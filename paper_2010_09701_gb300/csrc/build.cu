@@ -1570,10 +1570,11 @@ int build_hamiltonian(oefe_ctx* c, const double* veff, int store) {
   cudaStreamSynchronize(c->stream);
   dev_free(d_gw);
   if (st == OEFE_OK && (store & (OEFE_STORE_BF16X3 | OEFE_STORE_BF16X6))) {
-    // tensor maps of the split cell matrices, one per k-point
+    // tensor maps of the split cell matrices: per k-point one for whole tiles, one of 32-row boxes
     const size_t mb = tensor_map_bytes();
-    std::vector<unsigned char> maps(mb * c->kd.size());
-    for (size_t ik = 0; ik < c->kd.size() && st == OEFE_OK; ++ik) st = make_cell_tmap(c, c->kd[ik], maps.data() + ik * mb);
+    const size_t nk = c->kd.size();
+    std::vector<unsigned char> maps(2 * mb * nk);
+    for (size_t i = 0; i < 2 * nk && st == OEFE_OK; ++i) st = make_cell_tmap(c, c->kd[i / 2], i % 2 == 1, maps.data() + i * mb);
     if (st == OEFE_OK && c->n_tmaps != (int)c->kd.size()) {
       dev_free(c->d_tmaps);
       c->d_tmaps = nullptr;

@@ -420,7 +420,7 @@ int launch_cell_mma(oefe_ctx* c, const KData& K, const void* X, int ldx, int nv,
     k0.vblocks = (nv + 63) / 64;
     k0.tile0 = 0;
     const long long nt = (long long)c->ncells * k0.vblocks;
-    return launch_cell_mma_tma(c, (const char*)c->d_tmaps + (size_t)ik * tensor_map_bytes(), nullptr, &k0, 1, nt, cplx,
+    return launch_cell_mma_tma(c, (const char*)c->d_tmaps + (size_t)2 * ik * tensor_map_bytes(), nullptr, &k0, 1, nt, cplx,
                                K.bf_parts, (int)std::min<long long>(nt, c->num_sms), c->stream);
   }
   if (K.bf_parts != 2) { c->err = "tensor path: the split cell matrices have no tensor maps"; return OEFE_ERR_STATE; }

@@ -11,8 +11,8 @@
 //               part) into a ring of 32 KB shared-memory stages;
 //   warp 1      MMA issuer (one thread): waits for a full A stage (and B stage),
 //               issues the MMAs, commits to the stage's "empty" barriers;
-//   warps 2-5   gather producers: rows of X for every K tile, split to bf16;
-//   warps 6-9   epilogue: tensor memory -> registers -> per-cell products, one
+//   warps 2-5   (real data: 2-9) gather producers: rows of X for every K tile, split to bf16;
+//   four more   epilogue: tensor memory -> registers -> per-cell products, one
 //               M tile at a time, so the next tile's MMAs into an M tile start
 //               as soon as that M tile has been drained.
 // Every mbarrier wait is bounded; on a timeout the CTA raises the error flag,
@@ -34,7 +34,6 @@ namespace {
 constexpr int MT = 128;     // rows per M tile
 constexpr int KT = 64;      // K per tile (bf16: 128 bytes per row)
 constexpr int NBV = 64;     // vectors per tile (complex; real data also 128, the NVT parameter)
-constexpr int THREADS = 320;
 constexpr int MAXPAD = 4 * MT;  // largest npad
 
 // Shared-memory plan per (complex, bf16 parts): NPART planes per A stage (one part of the cell
@@ -44,6 +43,11 @@ template <bool CPLX, int NPART, int NVT = NBV>
 struct TmaCfg {
   static constexpr int SA = NPART == 2 ? 3 : 2;        // A ring stages
   static constexpr int SB = 2;                         // B ring stages
+  // groups of four gather warps, taking alternate K tiles: with 128-vector tiles of real data, whose
+  // matrices mostly come from L2, one group's loads are in flight while the other splits and stores;
+  // on complex data the stream of the matrices from memory sets the pace and a second group adds nothing
+  static constexpr int GG = CPLX ? 1 : 2;
+  static constexpr int THREADS = 192 + 128 * GG;
   static constexpr int ER = NPART == 2 ? 32 : 16;      // epilogue rows staged per round, per warp
   static constexpr int NB_ROWS = CPLX ? 2 * NBV : NVT;
   static constexpr int A_PLANE = MT * 128;
@@ -63,20 +67,21 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
-// barrier among the 128 gather threads (named barrier 1) that also ORs a flag over them, so that
+// barrier among the NT gather threads (named barrier 1) that also ORs a flag over them, so that
 // all of them take the same exit decision
+template <int NT>
 __device__ __forceinline__ bool gather_bar_or(bool v) {
   uint32_t r;
   asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, 128, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}\n"
       : "=r"(r)
-      : "r"((uint32_t)v)
+      : "r"((uint32_t)v), "n"(NT)
       : "memory");
   return r != 0;
 }
 
 struct TmaArgs {
-  const CUtensorMap* maps;  // one per k-point, in global memory
+  const CUtensorMap* maps;  // per k-point, in global memory: one for whole M tiles, one of 32-row boxes
   const MmaK* ks;           // per-k parameters in global memory, or null: use k0
   MmaK k0;
   int nk;
@@ -114,10 +119,25 @@ __device__ __forceinline__ void decode_tile(const TmaArgs& A, long long t, int* 
 // MERGE (complex only): the real part of the cell matrix multiplies [Re X | Im X] in one N = 128
 // MMA instead of two N = 64 ones (fewer tensor instructions; which is faster depends on the split,
 // so the autotuner chooses)
+// the staged rows to a block of odd width or its tail, a vector per lane
+template <bool CPLX, int ER>
+__device__ __forceinline__ void store_ragged(const unsigned char* st, float* z, int nrows, int v, int nv) {
+  constexpr int CPR = CPLX ? 16 : 8;
+  const int lane = threadIdx.x & 31, ch = CPLX ? lane >> 1 : lane >> 2, off = CPLX ? 8 * (lane & 1) : 4 * (lane & 3);
+  if (v >= nv) return;
+#pragma unroll 4
+  for (int rl = 0; rl < nrows; ++rl) {
+    const unsigned char* sp = st + rl * (CPR * 16) + ((ch ^ (rl & (CPR - 1))) << 4) + off;
+    float* zr = z + (size_t)rl * nv * (CPLX ? 2 : 1);
+    if (CPLX) reinterpret_cast<float2*>(zr)[v] = *reinterpret_cast<const float2*>(sp);
+    else zr[v] = *reinterpret_cast<const float*>(sp);
+  }
+}
+
 // NVT (real data only): vectors per tile, 64 or 128; with 128 a cell's matrix streams once for
-// twice the vectors (one N = 128 MMA per product, 128 tensor-memory columns per M tile)
+// twice the vectors (one N = 128 MMA per product, 128 tensor-memory columns per M tile).
 template <bool CPLX, int NPART, bool MERGE, int NVT = NBV>
-__global__ void __launch_bounds__(THREADS, 1) k_cell_mma_tma(const TmaArgs A) {
+__global__ void __launch_bounds__((TmaCfg<CPLX, NPART, NVT>::THREADS), 1) k_cell_mma_tma(const TmaArgs A) {
   static_assert(NVT == NBV || (!CPLX && NVT == 2 * NBV), "128-vector tiles are for real data");
   using Cfg = TmaCfg<CPLX, NPART, NVT>;
   constexpr int SA = Cfg::SA, SB = Cfg::SB, STG = Cfg::STG;
@@ -173,21 +193,35 @@ __global__ void __launch_bounds__(THREADS, 1) k_cell_mma_tma(const TmaArgs A) {
     // ---------------------------------------------------------------- TMA producer
     if (lane == 0) {
       long long ga = 0;
-      for (int k = 0; k < A.nk; ++k)
+      for (int k = 0; k < 2 * A.nk; ++k)
         asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&A.maps[k]) : "memory");
       for (long long t = blockIdx.x; t < A.ntiles && !s_fail; t += gridDim.x) {
         int k, e, vb, mte, kte;
         decode_tile(A, t, &k, &e, &vb);
         cell_tiles(A, e, mt, ktn, &mte, &kte);
+        const int naug = A.nloc + A.act_off[e + 1] - A.act_off[e];
         for (int it = 0; it < mte * kte * HALVES && !s_fail; ++it, ++ga) {
           const int h = it % HALVES, kt = it / (HALVES * mte), m = (it / HALVES) % mte;
           const int s = (int)(ga % SA);
           const long long u = ga / SA;
           if (u >= 1 && !mbar_wait(&a_empty[s], (uint32_t)((u - 1) & 1), &s_fail)) break;
-          mbar_expect_tx(&a_full[s], A_STAGE);
           // one contiguous block of NPART planes: (cell, K tile, M tile, real or imaginary part)
           const int chunk = ((e * ktn + kt) * mt + m) * HALVES + h;
-          tma_load_3d(smem_u32(sA + s * A_STAGE), &A.maps[k], 0, 0, NPART == 2 ? chunk : chunk * NPART, &a_full[s]);
+          const int n32 = (naug - m * MT + 31) / 32;
+          if (n32 >= 4) {
+            mbar_expect_tx(&a_full[s], A_STAGE);
+            tma_load_3d(smem_u32(sA + s * A_STAGE), &A.maps[2 * k], 0, 0, NPART == 2 ? chunk : chunk * NPART, &a_full[s]);
+          } else {
+            // the last M tile of a cell: only the 32-row boxes that hold rows of it (the rest of the
+            // stage is stale and feeds accumulator rows that nothing drains). At n_aug = 393 the
+            // padding of a fourth tile for 9 rows was a quarter of the bytes of a kernel that runs at
+            // four fifths of the memory's rate.
+            mbar_expect_tx(&a_full[s], NPART * n32 * 4096);
+            for (int p = 0; p < NPART; ++p)
+              for (int i = 0; i < n32; ++i)
+                tma_load_3d(smem_u32(sA + s * A_STAGE + p * A_PLANE + i * 4096), &A.maps[2 * k + 1], 0,
+                            NPART == 2 ? p * MT + 32 * i : 32 * i, NPART == 2 ? chunk : chunk * NPART + p, &a_full[s]);
+          }
         }
       }
       // drain: every issued load lands before the CTA leaves
@@ -270,9 +304,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_cell_mma_tma(const TmaArgs A) {
         mbar_wait_drain(&mma_done, 0);
       }
     }
-  } else if (warp < 6) {
+  } else if (warp < 2 + 4 * Cfg::GG) {
     // ---------------------------------------------------------------- gather producers
-    const int gt = tid - 64;  // 0 .. 127
+    const int gt = (tid - 64) & 127, group = (tid - 64) >> 7;
     long long gb = 0;
     int tg = 0;
     for (long long t = blockIdx.x; t < A.ntiles; t += gridDim.x) {
@@ -287,12 +321,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_cell_mma_tma(const TmaArgs A) {
       // the tile's row map, once per tile, double-buffered; the barrier publishes it and takes
       // the exit decision on a failure uniformly over the gather threads
       int* rows = s_rows[tg & 1];
-      for (int r = gt; r < naug; r += 128)
+      for (int r = tid - 64; r < naug; r += 128 * Cfg::GG)
         rows[r] = r < A.nloc ? A.cell_nodes[(size_t)e * A.nloc + r] : (int)(A.nh + A.act_idx[A.act_off[e] + r - A.nloc]);
       ++tg;
-      if (gather_bar_or(s_fail != 0)) break;
+      if (gather_bar_or<128 * Cfg::GG>(s_fail != 0)) break;
       for (int kt = 0; kt < kte && !s_fail; ++kt, ++gb) {
         const int sb = (int)(gb % SB);
+        if (Cfg::GG == 2 && sb != group) continue;
         const long long u = gb / SB;
         if (u >= 1 && !mbar_wait(&b_empty[sb], (uint32_t)((u - 1) & 1), &s_fail)) break;
         unsigned char* b0 = sB + sb * B_STAGE;
@@ -364,7 +399,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_cell_mma_tma(const TmaArgs A) {
       for (int m = 0; m < mte; ++m) {
         if (!mbar_wait(&acc_full[m], (uint32_t)(use[m] & 1), &s_fail)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int row = m * MT + 32 * q + lane;
         for (int h = 0; h < (CPLX ? 2 : NVT / 32); ++h) {
           const uint32_t tl0 = taddr + ((uint32_t)(32 * q) << 16) + m * MCOLS + 32 * h;
           float re[32], im[32];
@@ -372,10 +406,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_cell_mma_tma(const TmaArgs A) {
           if (CPLX) tmem_ld32(tl0 + NBV, im);
           const int vb0 = v0 + 32 * h;
           const bool full = CPLX ? ((P.nv & 1) == 0 && vb0 + 32 <= P.nv) : ((P.nv & 3) == 0 && vb0 + 32 <= P.nv);
-          if (full) {
-            // stage the warp's rows (ER at a time) x 32 values in shared memory (16-byte chunks,
-            // XOR-swizzled by row), then write whole row segments: 256 contiguous bytes per row
-            // (complex), 128 (real)
+          // stage the warp's rows (ER at a time) x 32 values in shared memory (16-byte chunks,
+          // XOR-swizzled by row), then write whole row segments: 256 contiguous bytes per row (complex),
+          // 128 (real); one vector per lane where the row's width or its tail allows no 16-byte stores
+          // (written straight from the registers, a row per lane, those blocks took three times as long)
+          {
             constexpr int CPR = CPLX ? 16 : 8;      // 16-byte chunks per row segment
             constexpr int RPI = 32 / CPR;           // rows per store instruction
             constexpr int ER = Cfg::ER;
@@ -392,33 +427,25 @@ __global__ void __launch_bounds__(THREADS, 1) k_cell_mma_tma(const TmaArgs A) {
                 }
               }
               __syncwarp();
-              const int ch = lane % CPR, rsub = lane / CPR;
+              const int row0 = m * MT + 32 * q + round * ER;
+              if (full) {
+                const int ch = lane % CPR, rsub = lane / CPR;
 #pragma unroll
-              for (int i = 0; i < ER; i += RPI) {
-                const int rl = i + rsub;                     // staging row
-                const int grow = m * MT + 32 * q + round * ER + rl;
-                if (rl < ER && grow < naug) {
-                  const float4 v =
-                      *reinterpret_cast<const float4*>(st + rl * (CPR * 16) + ((ch ^ (rl & (CPR - 1))) << 4));
-                  float* zr = P.Z + ((size_t)e * A.npad + grow) * (size_t)P.nv * (CPLX ? 2 : 1);
-                  *reinterpret_cast<float4*>(zr + (CPLX ? 2 : 1) * vb0 + 4 * ch) = v;
+                for (int i = 0; i < ER; i += RPI) {
+                  const int rl = i + rsub;                     // staging row
+                  const int grow = m * MT + 32 * q + round * ER + rl;   // (from row0 the unrolled addresses spill)
+                  if (rl < ER && grow < naug) {
+                    const float4 v =
+                        *reinterpret_cast<const float4*>(st + rl * (CPR * 16) + ((ch ^ (rl & (CPR - 1))) << 4));
+                    float* zr = P.Z + ((size_t)e * A.npad + grow) * (size_t)P.nv * (CPLX ? 2 : 1);
+                    *reinterpret_cast<float4*>(zr + (CPLX ? 2 : 1) * vb0 + 4 * ch) = v;
+                  }
                 }
+              } else {
+                store_ragged<CPLX, ER>(st, P.Z + ((size_t)e * A.npad + row0) * (size_t)P.nv * (CPLX ? 2 : 1), min(ER, naug - row0),
+                                       vb0 + lane, P.nv);
               }
               __syncwarp();
-            }
-          } else if (row < naug) {
-            float* zr = P.Z + ((size_t)e * A.npad + row) * (size_t)P.nv * (CPLX ? 2 : 1);
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const int v = vb0 + j;
-              if (v < P.nv) {
-                if (CPLX) {
-                  zr[2 * v] = re[j];
-                  zr[2 * v + 1] = im[j];
-                } else {
-                  zr[v] = re[j];
-                }
-              }
             }
           }
         }
@@ -459,7 +486,7 @@ size_t cell_mma_tma_smem(bool cplx, int parts, int nvt) {
 // Tensor map of one k-point's split cell matrices, stored tile-contiguous ([cell][K tile][M tile]
 // [plane][128][64]): one box = the bf16 parts of the real or of the imaginary part of one
 // (K tile, M tile).
-int make_cell_tmap(oefe_ctx* c, const KData& K, void* map_out) {
+int make_cell_tmap(oefe_ctx* c, const KData& K, bool rows32, void* map_out) {
   auto fn = encode_fn();
   if (!fn) { c->err = "cuTensorMapEncodeTiled is not available"; return OEFE_ERR_CUDA; }
   const int parts = K.bf_parts;
@@ -467,10 +494,10 @@ int make_cell_tmap(oefe_ctx* c, const KData& K, void* map_out) {
   const int planes = (K.cplx ? 2 : 1) * parts;
   const cuuint64_t nplanes = (cuuint64_t)c->ncells * (c->npad / KT) * (c->npad / MT) * planes;
   // two parts: (column, row of a plane pair, chunk), box (64, 256, 1); three parts: (column, row,
-  // plane), box (64, 128, 3) (a box dimension holds at most 256)
+  // plane), box (64, 128, 3) (a box dimension holds at most 256); rows32: boxes of 32 rows of a plane
   const cuuint64_t dims[3] = {(cuuint64_t)KT, (cuuint64_t)MT * (parts == 2 ? 2 : 1), parts == 2 ? nplanes / 2 : nplanes};
   const cuuint64_t strides[2] = {(cuuint64_t)KT * 2, (cuuint64_t)MT * KT * 2 * (parts == 2 ? 2 : 1)};
-  const cuuint32_t box[3] = {KT, (cuuint32_t)MT * (parts == 2 ? 2 : 1), parts == 2 ? 1u : 3u};
+  const cuuint32_t box[3] = {KT, rows32 ? 32u : (cuuint32_t)MT * (parts == 2 ? 2 : 1), rows32 || parts == 2 ? 1u : 3u};
   const cuuint32_t estr[3] = {1, 1, 1};
   CUtensorMap m;
   const CUresult r = fn(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, K.Hbf, dims, strides, box, estr,
@@ -510,7 +537,7 @@ int launch_cell_mma_tma(oefe_ctx* c, const void* d_maps, const MmaK* d_ks, const
   const size_t smem = cell_mma_tma_smem(cplx, parts, nvt);
   auto go = [&](auto kern) -> int {
     OEFE_CUDA_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    OEFE_COUNTED kern<<<grid, THREADS, smem, st>>>(A);
+    OEFE_COUNTED kern<<<grid, cplx ? TmaCfg<true, 2>::THREADS : TmaCfg<false, 2>::THREADS, smem, st>>>(A);
     return OEFE_OK;
   };
   // merged real-part MMAs: the tuned choice, else on (measured faster for both splits)

@@ -11,6 +11,7 @@
 #include <cmath>
 
 #include "oefe_internal.h"
+#include "pair_int_dev.cuh"
 
 namespace {
 
@@ -196,6 +197,13 @@ __global__ void k_node_update(const typename Sc<T, C>::type* __restrict__ Z, con
 constexpr int ER_T = 1024;
 constexpr int ER_SC = 2048;
 
+__device__ __forceinline__ double widen(float x) { return widen_int(x); }
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// Each CTA takes one of gridDim.z equal column groups of at most ER_V vectors: more CTAs than one per
+// function, so that the last wave is short (310 functions on 304 resident CTAs took two waves). The
+// slot groups, so the order of a sum, are those of a pass over that group alone.
+constexpr int ER_V = 128;
 template <typename S, bool C>
 __device__ __forceinline__ void enr_reduce_cta(const S* __restrict__ Z, int nv, int64_t s0, int64_t s1,
                                                const int64_t* __restrict__ enr_slot, cd* __restrict__ yo) {
@@ -203,16 +211,19 @@ __device__ __forceinline__ void enr_reduce_cta(const S* __restrict__ Z, int nv, 
   __shared__ int64_t off[ER_SC];
   constexpr int NW = ER_T / 32;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int nvc = (nv + 31) / 32;
+  const int v0 = (int)((long long)blockIdx.z * nv / gridDim.z), v1 = (int)((blockIdx.z + 1LL) * nv / gridDim.z);
+  const int nvc = (v1 - v0 + 31) / 32;
   for (int vc0 = 0; vc0 < nvc; vc0 += NW) {
     const int nc = min(NW, nvc - vc0);   // vector chunks of this pass
     const int G = NW / nc;               // slot groups
-    const int g = w / nc, v = (vc0 + w % nc) * 32 + lane;
-    const bool active = g < G && v < nv;
+    const int g = w / nc, v = v0 + (vc0 + w % nc) * 32 + lane;
+    const bool active = g < G && v < v1;
     double sx = 0, sy = 0;
+    // FP32 products widen on the integer pipe: the conversion instruction would take as long on the
+    // FP64 pipe, which bounds this sum, as the addition itself
     auto add = [&](const S z) {
-      if constexpr (C) { sx += (double)z.x; sy += (double)z.y; }
-      else sx += (double)z;
+      if constexpr (C) { sx += widen(z.x); sy += widen(z.y); }
+      else sx += widen(z);
     };
     for (int64_t c0 = s0; c0 < s1; c0 += ER_SC) {   // the same trip count in every thread
       const int m = (int)min((int64_t)ER_SC, s1 - c0);
@@ -240,7 +251,7 @@ __device__ __forceinline__ void enr_reduce_cta(const S* __restrict__ Z, int nv, 
         ax += r.x;
         ay += r.y;
       }
-      if (v < nv) yo[v] = mkc(ax, ay);
+      if (v < v1) yo[v] = mkc(ax, ay);
     }
     __syncthreads();
   }
@@ -315,8 +326,69 @@ struct NodeK {
 // overlap (the slot indices are warp-uniform broadcast loads); rows whose width and leading
 // dimensions allow it move as float4. Complex rows are handled as interleaved reals (every
 // operation here is componentwise). The recurrence runs in the filter's precision.
-template <typename T, bool C>
-__global__ void __launch_bounds__(256) k_node_update_multi(const NodeK* __restrict__ P,
+// One node row in vectors VT of a lane, SG of them at a time, so that the rows of all of them are in flight
+// together; product rows in ascending slot order.
+template <typename VT, int SG, int R, typename T>
+__device__ __forceinline__ void node_row(const NodeK& p, const T* Zt, const int64_t* slots, int ns, int64_t g, int W, int ldk,
+                                         int ldm1, int ldy, int ldr, float minv, bool has_k, bool has_m1, bool has_r) {
+  constexpr int N = sizeof(VT) / sizeof(float);
+  const float* Z = (const float*)Zt;
+  const float alpha = (float)p.alpha, cs = (float)p.cshift, beta = (float)p.beta;
+  auto ld = [](const float* q, float (&v)[N]) {
+    const VT x = *reinterpret_cast<const VT*>(q);
+#pragma unroll
+    for (int c = 0; c < N; ++c) v[c] = reinterpret_cast<const float*>(&x)[c];
+  };
+  for (int f0 = N * (threadIdx.x & 31); f0 < W; f0 += 32 * N * SG) {
+    float acc[SG][N], xk[SG][N], xm[SG][N], rr[SG][N];
+#pragma unroll
+    for (int i = 0; i < SG; ++i) {
+      const int f = f0 + 32 * N * i;
+#pragma unroll
+      for (int c = 0; c < N; ++c) acc[i][c] = xk[i][c] = xm[i][c] = rr[i][c] = 0.f;
+      if (f < W && has_k) ld((const float*)p.Xk + g * ldk + f, xk[i]);
+      if (f < W && has_m1) ld((const float*)p.Xm1 + g * ldm1 + f, xm[i]);
+      if (f < W && has_r) ld((const float*)p.R + g * ldr + f, rr[i]);
+    }
+    for (int s2 = 0; s2 < ns; s2 += 2) {
+      const int64_t sa = slots[s2], sb = s2 + 1 < ns ? slots[s2 + 1] : -1;
+      float za[SG][N], zb[SG][N];
+#pragma unroll
+      for (int i = 0; i < SG; ++i) {
+        const int f = f0 + 32 * N * i;
+#pragma unroll
+        for (int c = 0; c < N; ++c) za[i][c] = zb[i][c] = 0.f;
+        if (f < W) ld(Z + sa * W + f, za[i]);
+        if (f < W && sb >= 0) ld(Z + sb * W + f, zb[i]);
+      }
+#pragma unroll
+      for (int i = 0; i < SG; ++i)
+#pragma unroll
+        for (int c = 0; c < N; ++c) acc[i][c] = acc[i][c] + za[i][c] + zb[i][c];
+    }
+#pragma unroll
+    for (int i = 0; i < SG; ++i) {
+      const int f = f0 + 32 * N * i;
+      if (f >= W) continue;
+      VT o;
+#pragma unroll
+      for (int c = 0; c < N; ++c) {
+        float v = alpha * (acc[i][c] * minv - cs * xk[i][c]);
+        if (has_m1) v += beta * xm[i][c];
+        if (has_r) v += alpha * p.coef[(f + c) / R] * rr[i][c];   // component f + c belongs to vector (f + c) / R
+        reinterpret_cast<float*>(&o)[c] = v;
+      }
+      *reinterpret_cast<VT*>((float*)p.Y + g * ldy + f) = o;
+    }
+  }
+}
+
+// WIDE: rows of more than 128 reals take three float4 per lane at a time, rows that allow only 8-byte
+// accesses (an odd number of complex vectors) four float2; a block with either in a pass takes this
+// instance. Its own instance, since its registers would cost the narrow rows a third of their warps in
+// flight (126 -> 216 us a degree of two blocks of 64 complex vectors).
+template <typename T, bool C, bool WIDE>
+__global__ void __launch_bounds__(256, WIDE ? 0 : 5) k_node_update_multi(const NodeK* __restrict__ P,
                                                            const int64_t* __restrict__ node_off,
                                                            const int64_t* __restrict__ node_slot,
                                                            const double* __restrict__ m, int64_t nh) {
@@ -341,7 +413,12 @@ __global__ void __launch_bounds__(256) k_node_update_multi(const NodeK* __restri
                    (!has_k || (ldk % 4 == 0 && ((uintptr_t)Xk & 15) == 0)) &&
                    (!has_m1 || (ldm1 % 4 == 0 && ((uintptr_t)Xm1 & 15) == 0)) &&
                    (!has_r || (ldr % 4 == 0 && ((uintptr_t)Rr & 15) == 0));
-  if (vec && W <= 128) {
+  // rows whose width or alignment allows only 8-byte accesses (an odd number of complex vectors)
+  const bool vec2 = sizeof(T) == 4 && W % 2 == 0 && ldy % 2 == 0 && ((uintptr_t)Y & 7) == 0 &&
+                    (!has_z || ((uintptr_t)Z & 7) == 0) && (!has_k || (ldk % 2 == 0 && ((uintptr_t)Xk & 7) == 0)) &&
+                    (!has_m1 || (ldm1 % 2 == 0 && ((uintptr_t)Xm1 & 7) == 0)) &&
+                    (!has_r || (ldr % 2 == 0 && ((uintptr_t)Rr & 7) == 0));
+  if (!WIDE && vec && W <= 128) {
     // one float4 per lane covers a row: two nodes per pass of the warp, so that the dependent loads
     // of the two (slot range, slot indices, product rows) overlap; per node the same operations in
     // the same order as the general loop below
@@ -417,50 +494,10 @@ __global__ void __launch_bounds__(256) k_node_update_multi(const NodeK* __restri
     const int64_t s0 = node_off[g];
     const int ns = has_z ? (int)(node_off[g + 1] - s0) : 0;
     const T minv = (T)(1.0 / m[g]);
-    if (vec) {
-      for (int f = 4 * lane; f < W; f += 128) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int s8 = 0; s8 < ns; s8 += 8) {
-          // slot indices: the same address in every lane (one broadcast load each), then the rows
-          int64_t sl[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) sl[u] = s8 + u < ns ? node_slot[s0 + s8 + u] : 0;
-          float4 z[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u)
-            z[u] = s8 + u < ns ? *reinterpret_cast<const float4*>((const float*)Z + sl[u] * W + f)
-                               : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            acc.x += z[u].x;
-            acc.y += z[u].y;
-            acc.z += z[u].z;
-            acc.w += z[u].w;
-          }
-        }
-        const float4 xk = has_k ? *reinterpret_cast<const float4*>((const float*)Xk + g * ldk + f)
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 o;
-        o.x = (float)alpha * (acc.x * (float)minv - (float)cs * xk.x);
-        o.y = (float)alpha * (acc.y * (float)minv - (float)cs * xk.y);
-        o.z = (float)alpha * (acc.z * (float)minv - (float)cs * xk.z);
-        o.w = (float)alpha * (acc.w * (float)minv - (float)cs * xk.w);
-        if (has_m1) {
-          const float4 xm = *reinterpret_cast<const float4*>((const float*)Xm1 + g * ldm1 + f);
-          o.x += (float)beta * xm.x;
-          o.y += (float)beta * xm.y;
-          o.z += (float)beta * xm.z;
-          o.w += (float)beta * xm.w;
-        }
-        if (has_r) {   // component f + i belongs to vector (f + i) / R
-          const float4 r = *reinterpret_cast<const float4*>((const float*)Rr + g * ldr + f);
-          o.x += (float)alpha * coef[(f + 0) / R] * r.x;
-          o.y += (float)alpha * coef[(f + 1) / R] * r.y;
-          o.z += (float)alpha * coef[(f + 2) / R] * r.z;
-          o.w += (float)alpha * coef[(f + 3) / R] * r.w;
-        }
-        *reinterpret_cast<float4*>((float*)Y + g * ldy + f) = o;
-      }
+    if (WIDE && vec) {
+      node_row<float4, 3, R>(p, Z, node_slot + s0, ns, g, W, ldk, ldm1, ldy, ldr, (float)minv, has_k, has_m1, has_r);
+    } else if (WIDE && vec2) {
+      node_row<float2, 4, R>(p, Z, node_slot + s0, ns, g, W, ldk, ldm1, ldy, ldr, (float)minv, has_k, has_m1, has_r);
     } else {
       for (int f = lane; f < W; f += 32) {
         T acc = T(0);
@@ -493,6 +530,7 @@ __global__ void k_enr_update_multi(const NodeK* __restrict__ P, int nO, int64_t 
   const int nu = t / p.nv, v = t % p.nv;
   cd s = mkc(0, 0);
   if (p.Z) {   // no products at the first degree of the defect recurrence
+#pragma unroll 8
     for (int mu = 0; mu < nO; ++mu) {
       const cd yo = p.Yo[mu * p.nv + v];
       if constexpr (C) s += reinterpret_cast<const cd*>(p.Minv)[nu * nO + mu] * yo;
@@ -572,14 +610,14 @@ struct Step {
 };
 
 // Rows per CTA of the dense cell products: a CTA takes every row of its cell and vector block when
-// those blocks fill the GPU twice over, else the rows are shared out (multiples of 16, one pass of
-// the warps) until they do. Each row's sum is the same either way. The two-atom cell has 16 refined
+// those blocks fill the GPU six times over (a last wave that is nearly empty then costs little), else
+// the rows are shared out (multiples of 16, one pass of the warps) until they do. Each row's sum is the same either way. The two-atom cell has 16 refined
 // cells, so 16 CTAs: 183 us a product of 20 real vectors, 757 us of 13 complex ones.
 int dense_rows_per_cta(const oefe_ctx* c, long long blocks) {
-  const int most = (c->npad + 15) / 16;
-  const long long want = (2LL * c->num_sms + blocks - 1) / std::max(blocks, 1LL);
+  const int most = (c->npad + 7) / 8;
+  const long long want = (6LL * c->num_sms + blocks - 1) / std::max(blocks, 1LL);
   const int nz = (int)std::max(1LL, std::min<long long>(want, most));
-  return ((c->npad + nz - 1) / nz + 15) / 16 * 16;
+  return ((c->npad + nz - 1) / nz + 7) / 8 * 8;
 }
 
 template <typename T, bool C>
@@ -626,7 +664,7 @@ int launch_step(oefe_ctx* c, const KData& K, int dtype, const void* Hm, const vo
                                                      (const S*)Xm1, ldm1, (S*)Y, ldy);
   if (c->nO > 0) {
     const int eb = (c->nO * nv + 127) / 128;
-    OEFE_COUNTED k_enr_reduce<T, C><<<c->nO, ER_T, 0, c->stream>>>((const S*)Zbuf, c->d_enr_off, c->d_enr_slot, nv, Yo);
+    OEFE_COUNTED k_enr_reduce<T, C><<<dim3(c->nO, 1, (nv + ER_V - 1) / ER_V), ER_T, 0, c->stream>>>((const S*)Zbuf, c->d_enr_off, c->d_enr_slot, nv, Yo);
     OEFE_COUNTED k_enr_update<T, C><<<eb, 128, 0, c->stream>>>(Yo, K.Mooinv, c->nO, nv, c->nh, st.mode, st.alpha, st.cshift,
                                                   st.beta, (const S*)Xk, ldk, (const S*)Xm1, ldm1, (S*)Y, ldy);
   }
@@ -878,10 +916,18 @@ int batched_launch_degrees(oefe_ctx* c, const BatchPlan& P, bool cplx, const Mma
       }
     }
     if (timed) cudaEventRecordWithFlags(c->bev_kernel[2 * j + 1], c->bstream, cudaEventRecordExternal);
-    dim3 g1(nblocks, P.nk), g2(std::max(eb, 1), P.nk), gr(std::max(c->nO, 1), P.nk);
+    dim3 g1(nblocks, P.nk), g2(std::max(eb, 1), P.nk), gr(std::max(c->nO, 1), P.nk, (vmax + ER_V - 1) / ER_V);
+    bool wide = false;   // some block's rows are not those of the narrow instance
+    for (int k = 0; k < P.nk; ++k) {
+      const int W = P.nd[k].nv * (cplx ? 2 : 1);
+      wide = wide || W > 128 || W % 4 != 0;
+    }
+    auto node = [&](auto kern) {
+      OEFE_COUNTED kern<<<g1, 256, 0, c->bstream>>>(d_nd + (size_t)j * P.nk, c->d_node_off, c->d_node_slot, c->d_m, c->nh);
+    };
     if (cplx) {
-      OEFE_COUNTED k_node_update_multi<float, true><<<g1, 256, 0, c->bstream>>>(d_nd + (size_t)j * P.nk, c->d_node_off, c->d_node_slot,
-                                                                   c->d_m, c->nh);
+      if (wide) node(k_node_update_multi<float, true, true>);
+      else node(k_node_update_multi<float, true, false>);
       if (c->nO > 0) {
         if (product)
           OEFE_COUNTED k_enr_reduce_multi<float, true><<<gr, ER_T, 0, c->bstream>>>(d_nd + (size_t)j * P.nk, c->d_enr_off,
@@ -889,8 +935,8 @@ int batched_launch_degrees(oefe_ctx* c, const BatchPlan& P, bool cplx, const Mma
         OEFE_COUNTED k_enr_update_multi<float, true><<<g2, 128, 0, c->bstream>>>(d_nd + (size_t)j * P.nk, c->nO, c->nh);
       }
     } else {
-      OEFE_COUNTED k_node_update_multi<float, false><<<g1, 256, 0, c->bstream>>>(d_nd + (size_t)j * P.nk, c->d_node_off,
-                                                                    c->d_node_slot, c->d_m, c->nh);
+      if (wide) node(k_node_update_multi<float, false, true>);
+      else node(k_node_update_multi<float, false, false>);
       if (c->nO > 0) {
         if (product)
           OEFE_COUNTED k_enr_reduce_multi<float, false><<<gr, ER_T, 0, c->bstream>>>(d_nd + (size_t)j * P.nk, c->d_enr_off,
@@ -1282,8 +1328,23 @@ namespace {
 
 // vectors per k-point of one batched pass: wider blocks run as several passes over column groups
 // (the columns of the filter are independent), which bounds the per-cell products and recurrence
-// buffers; each group keeps its own captured graph
+// buffers; each group keeps its own captured graph. A pass of every column streams the cell matrices
+// once (the tiles of one cell's vector blocks are neighbours in the launch order, so all but the first
+// read them from L2), so every column goes in one pass when its buffers take at most 1 / FILTER_WS_SHARE
+// of the device's memory, else groups of FILTER_CHUNK: 360 real columns on the 16^3 supercell (12 GB)
+// take one pass instead of three, on the 32^3 one (95 GB) three.
 constexpr int FILTER_CHUNK = 128;
+constexpr int FILTER_WS_SHARE = 8;
+
+int filter_groups(const oefe_ctx* c, int nk, const int* nv, int vmax, int dtype) {
+  const int most = (vmax + FILTER_CHUNK - 1) / FILTER_CHUNK;
+  if (most == 1) return 1;
+  const double es = (double)dtype_bytes(dtype), es_low = dtype_complex(dtype) ? 8.0 : 4.0, n = (double)(c->nh + c->nO);
+  const double per = (double)c->ncells * c->npad * es_low + n * (3.0 * es_low + (dtype_fp64(dtype) ? 2.0 * es : 0.0));
+  double bytes = 0;
+  for (int k = 0; k < nk; ++k) bytes += (double)nv[k] * per;
+  return bytes * FILTER_WS_SHARE <= (double)c->dev_bytes ? 1 : most;
+}
 
 int filter_batched_groups(oefe_ctx* c, int nk, void* const* X, const int* nv, const int* ld, int dtype, int degree,
                           const double* a, const double* b, const double* a0, const double* theta, int flags) {
@@ -1293,7 +1354,7 @@ int filter_batched_groups(oefe_ctx* c, int nk, void* const* X, const int* nv, co
     ok = nv[k] >= 1;
     vmax = std::max(vmax, ok ? nv[k] : 0);
   }
-  const int Q = (vmax + FILTER_CHUNK - 1) / FILTER_CHUNK;
+  const int Q = ok && dtype >= 0 && dtype <= 3 ? filter_groups(c, nk, nv, vmax, dtype) : 1;
   for (int k = 0; ok && k < nk; ++k) ok = nv[k] >= Q;
   if (!ok || Q <= 1 || dtype < 0 || dtype > 3)   // one pass (the call checks its arguments itself)
     return filter_batched_impl(c, nk, X, nv, ld, dtype, degree, a, b, a0, theta, flags);

@@ -302,7 +302,7 @@ double fp64_product_flops(const oefe_ctx* c, bool cplx, int nv);
 void gauss_rule(int n, std::vector<double>& x, std::vector<double>& w);
 int launch_cell_mma_tma(oefe_ctx* c, const void* d_maps, const MmaK* d_ks, const MmaK* k0, int nk, long long ntiles,
                         bool cplx, int parts, int grid, cudaStream_t st, int nvt = 64);
-int make_cell_tmap(oefe_ctx* c, const KData& K, void* map_out);
+int make_cell_tmap(oefe_ctx* c, const KData& K, bool rows32, void* map_out);
 size_t tensor_map_bytes();
 size_t cell_mma_tma_smem(bool cplx, int parts, int nvt = 64);
 int launch_cell_mma_ptrs(oefe_ctx* c, const void* H, const void* X, int ldx, int nv, void* Z, bool cplx, int nb,
