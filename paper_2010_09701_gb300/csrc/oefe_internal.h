@@ -204,6 +204,7 @@ struct oefe_ctx {
   int* d_sf_index = nullptr;            // cell -> row of d_sf, or -1
   int* d_dense_index = nullptr;         // cell -> position in d_dense_cells, or -1
   int n_sf = 0, n_dense = 0, sf_nbuf = 0;
+  std::vector<int> sf_n1_h;             // points per axis of the sum-factorization list's cells (ascending)
   double* d_veff = nullptr;             // V_eff at the points of the last operator build
   int tune_merge = -1;                  // TMA kernel: merged real-part MMAs (1), separate (0), untuned (-1)
   double tune_ms[6] = {0, 0, 0, 0, 0, 0};
@@ -297,6 +298,8 @@ int setup_sumfac(oefe_ctx* c);
 bool sumfac_ready(const oefe_ctx* c);
 int launch_cell_apply_sf(oefe_ctx* c, const KData& K, const void* X, int ldx, int nv, bool cplx, void* Z,
                          cudaStream_t st);
+// the same in pairs, for the orders and rules with register-tiled kernels (sumfac_pair.cu)
+int launch_sf_pair(oefe_ctx* c, const KData& K, const void* X, int ldx, int nv, bool cplx, void* Z, bool* done, cudaStream_t st);
 void cell_box(const oefe_ctx* c, int e, double lo[3], double hi[3]);
 double fp64_product_flops(const oefe_ctx* c, bool cplx, int nv);
 void gauss_rule(int n, std::vector<double>& x, std::vector<double>& w);

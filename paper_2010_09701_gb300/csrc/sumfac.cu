@@ -275,9 +275,17 @@ int setup_sumfac(oefe_ctx* c) {
   std::vector<double> gx[13], gw[13];
   for (int e = 0; e < c->ncells; ++e) {
     const int l0 = c->leaf_off[e], l1 = c->leaf_off[e + 1];
-    const Leaf& L = c->leaves[l0];
-    if (l1 - l0 != 1 || L.n1 > SF_MAXN1) { den.push_back(e); continue; }
+    if (l1 - l0 != 1 || c->leaves[l0].n1 > SF_MAXN1) den.push_back(e);
+    else sfc.push_back(e);
+  }
+  // cells with the same rule next to each other: one launch per rule (pair products)
+  std::stable_sort(sfc.begin(), sfc.end(),
+                   [&](int x, int y) { return c->leaves[c->leaf_off[x]].n1 < c->leaves[c->leaf_off[y]].n1; });
+  c->sf_n1_h.clear();
+  for (int e : sfc) {
+    const Leaf& L = c->leaves[c->leaf_off[e]];
     const int n1 = L.n1;
+    c->sf_n1_h.push_back(n1);
     if (gw[n1].empty()) gauss_rule(n1, gx[n1], gw[n1]);
     n1max = std::max(n1max, n1);
     double lo[3], hi[3];
@@ -314,7 +322,6 @@ int setup_sumfac(oefe_ctx* c) {
           t[SF_A + o] = g1 - g2;
         }
     }
-    sfc.push_back(e);
     tabs.insert(tabs.end(), t.begin(), t.end());
   }
   // work buffers: every intermediate of the contractions (n1 may be below P) and two P^3 blocks
@@ -382,6 +389,10 @@ int launch_cell_apply_sf(oefe_ctx* c, const KData& K, const void* X, int ldx, in
   };
   if (c->f64_products == OEFE_F64_PAIRS) {
     if (!K.Hp) { c->err = "FP32-pair products: build the operator with OEFE_STORE_F64PAIR"; return OEFE_ERR_STATE; }
+    // register-tiled kernels for the orders and rules in use (half the time of the general kernel below)
+    bool done = false;
+    OEFE_TRY(launch_sf_pair(c, K, X, ldx, nv, cplx, Z, &done, st));
+    if (done) return OEFE_OK;
     // launch shapes: one CTA of 512 threads per SM over 4 (complex) vectors, or two CTAs of 384 or
     // of 512 threads per SM over 2 vectors each (half the shared memory, the cell's enrichment
     // blocks read twice as often); the fastest on this operator is kept after timing each once
