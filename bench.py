@@ -48,15 +48,9 @@ TRAFFIC_TENSOR = {   # bf16 parts of the split -> DRAM bytes per (k, cell, 64-ve
     3: {"bytes_per_tile": (3.064588e9 + 0.008374e9) / 1728, "source": "profiles/k_cell_mma_tma_c3mid_12cube_p6.md"},
 }
 TRAFFIC_FP64 = None   # {"bytes_per_cell", "source"} from a capture of the current FP64 product kernels
-# the FP64-class products in pair mode, real data: DRAM bytes of the sum-factorized kernel per launch
-# of 64 columns and single-leaf cell, from the capture of the current kernel on the 16^3 supercell
-# (3600 single-leaf cells; eight vectors per CTA there); the refined cells' dense product is not in it.
-# Complex data has no capture of the current kernel (the one of the small zincblende cell predates the
-# chunk-major enrichment rows), so its traffic is reported as unknown.
-TRAFFIC_PAIR = {"sf_bytes_per_cell": (2.167341e9 + 0.736962e9) / 3600,
-                "source": ("profiles/fp64_class_product_fields_wide_c5mid_16cube_p6.md: k_cell_apply_sf DRAM bytes "
-                           "per single-leaf cell, scaled by the single-leaf cells; the refined cells' dense product "
-                           "not included")}
+# the FP64-class products in pair mode: DRAM bytes of the single-leaf cells' kernels per launch of 64 columns and
+# cell, {"sf_bytes_per_cell", "source"} from a capture of the current kernels
+TRAFFIC_PAIR = None
 
 
 def is_complex(w):
@@ -427,8 +421,9 @@ def run_ours(args, rank, world):
     s_per_pass = float(np.mean(filt_ms)) * 1e-3 / (nk if batched else 1)
     # dominant kernel: the FP32 (complex64) cell product
     per_launch_ms = kms / max(klaunch, 1)
-    # a batched launch covers every k-point and one group of at most 128 vectors per k
-    ngroups = -(-max(nvs) // 128)
+    # a batched launch covers every k-point and one column group (all columns when they fit the filter's share of
+    # the device memory, else at most 128 per k): one launch per degree but the last and group
+    ngroups = min(-(-max(nvs) // 128), max(1, round(klaunch / max(args.steps * (deg - 1), 1))))
     nv_launch = [-(-v // ngroups) for v in nvs] if batched else nvs[:1]
     kflops = sum(kernel_flops_per_launch(naug, v, cplx) for v in nv_launch)
     nparts = 2 if bf16x3 else 3                # bf16 parts per real value of the split matrices
@@ -587,7 +582,7 @@ def run_ours(args, rank, world):
         if pairs:
             # the refined cells (dense FP64) take a few percent of the launch; the peak is that of
             # the pair arithmetic on the FP32 pipe
-            kname = ("k_cell_apply_sf<f2> + %s (FP64-class cell products: sum factorization in "
+            kname = ("k_sf_cc + k_sf_strips + %s (FP64-class cell products: sum factorization in "
                      "FP32-pair arithmetic on single-leaf cells, FP64 dense on the refined cells)"
                      % ("k_cell_apply_z3" if cplx else "k_cell_apply<double>"))
             peak, psrc = PAIR_PEAK_DERIVED, "derived: 152 SM x 128 FP32 lanes x 2070 MHz / 12 per pair FMA x 2 flops"

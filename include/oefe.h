@@ -361,7 +361,7 @@ int oefe_kernel_time(oefe_ctx_t ctx, double* ms, int64_t* launches);
 
 /* oefe_release_workspace -- frees the context's cached scratch (the growable
  * work arrays of the operator build, the filter and the subspace calls, among
- * them the digit planes of the tensor-core Gram matrices and rotations) and
+ * them the digit planes and partial sums of the tensor-core Gram matrices and rotations) and
  * the captured graph of the batched filter, which points into it; later calls
  * allocate what they need again. Synchronizes the context's streams. Returns
  * OEFE_ERR_ARG for a null context. No counterpart in the paper (memory
@@ -394,11 +394,14 @@ int oefe_launch_count(int64_t* n);
  *     oefe_rayleigh_ritz; refined cells stay FP64), the per-V operator build,
  *     the fields of oefe_density / oefe_band_trace_grad and the Jacobi sweeps
  *     of the projected eigenproblem;
- *   - tensor-core GEMMs with exact bf16 digits (7 digits of 7 bits per value,
- *     exact FP32 accumulation, about 2^-46 of the row and column maxima per
- *     term) for the Gram matrices and rotations of oefe_orthonormalize and
- *     oefe_rayleigh_ritz (digits cut into planes for nv <= 64, inside the MMA
- *     kernels for wider blocks).
+ *   - tensor-core GEMMs with exact bf16 digits (exact FP32 accumulation) for the
+ *     Gram matrices and rotations of oefe_orthonormalize and oefe_rayleigh_ritz:
+ *     7 digits of 7 bits per value, about 2^-46 of the row and column maxima
+ *     per term (digits cut into planes for nv <= 64, inside the MMA kernel for
+ *     the projected matrices of wider blocks), and 8 balanced digits, about
+ *     2^-53, for the Gram matrices of oefe_orthonormalize and every rotation of
+ *     wider blocks; 8 digits also for the enrichment part of the fields where
+ *     the rules have p + 1 and p + 3 points and p is 3 to 6.
  * Inputs and outputs stay FP64; Cholesky factors, triangular inverses and the
  * setup stay FP64. The operator must be built with OEFE_STORE_F64PAIR in pair
  * mode, else the products return OEFE_ERR_STATE; the build after the switch
@@ -407,8 +410,10 @@ int oefe_launch_count(int64_t* n);
 int oefe_set_f64_products(oefe_ctx_t ctx, int mode);
 
 /* oefe_set_product_shape -- launch shape of the FP32-pair cell products of the
- * single-leaf cells. shape -1 (default): each shape is timed once at the first
- * pair product of the context and the fastest is kept; 0: 4 complex (8 real)
+ * single-leaf cells where the register-tiled kernels do not apply (p outside 3
+ * to 6, or a cell with neither p + 1 nor p + 3 points per axis). shape -1
+ * (default): each shape is timed once at the first such product of the
+ * context and the fastest is kept; 0: 4 complex (8 real)
  * vectors per CTA of 512 threads; 1: 2 complex (4 real) vectors per CTA of
  * 384 threads; 2: 2 complex (4 real) vectors per CTA of 512 threads. Every
  * shape computes the same numbers. Returns OEFE_ERR_ARG for another value. */
