@@ -20,7 +20,7 @@ static void free_all(oefe_ctx* c) {
     dev_free(K.E0); dev_free(K.NO); dev_free(K.NOp);
   }
   c->kd.clear();
-  void* ptrs[] = {c->d_gll, c->d_m, c->d_cell_nodes, c->d_cellbox, c->d_pos, c->d_lm, c->d_R, c->d_dR,
+  void* ptrs[] = {c->d_gll, c->d_m, c->d_minv, c->d_cell_nodes, c->d_cellbox, c->d_pos, c->d_lm, c->d_R, c->d_dR,
                   c->d_act_off, c->d_act_idx, c->d_node_off, c->d_node_slot, c->d_enr_off, c->d_enr_slot,
                   c->d_qxyz, c->d_qw, c->d_leaves, c->d_leaf_off, c->d_q_off, c->d_dblk, c->ws, c->ws2,
                   c->d_status};

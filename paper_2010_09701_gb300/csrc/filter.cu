@@ -315,6 +315,7 @@ struct NodeK {
   const void* Minv;
   int ldk, ldm1, ldy, nv, mode;
   double alpha, cshift, beta;
+  float falpha, fcshift, fbeta;   // rounded here: a conversion per thread runs on the FP64 pipe
   // defect recurrence: Y += alpha coef[v] R[:, v] (R null: no addend)
   const void* R;
   const float* coef;
@@ -333,7 +334,7 @@ __device__ __forceinline__ void node_row(const NodeK& p, const T* Zt, const int6
                                          int ldm1, int ldy, int ldr, float minv, bool has_k, bool has_m1, bool has_r) {
   constexpr int N = sizeof(VT) / sizeof(float);
   const float* Z = (const float*)Zt;
-  const float alpha = (float)p.alpha, cs = (float)p.cshift, beta = (float)p.beta;
+  const float alpha = p.falpha, cs = p.fcshift, beta = p.fbeta;
   auto ld = [](const float* q, float (&v)[N]) {
     const VT x = *reinterpret_cast<const VT*>(q);
 #pragma unroll
@@ -383,6 +384,9 @@ __device__ __forceinline__ void node_row(const NodeK& p, const T* Zt, const int6
   }
 }
 
+// minv_of: the reciprocal masses, rounded from FP64 once per mesh. A division per row and lane kept the FP64
+// pipe 72% busy and set the pace of narrow rows (two blocks of 64
+// complex vectors on the 8-atom cell: 30 degrees 14.3 -> 13.7 ms).
 // WIDE: rows of more than 128 reals take three float4 per lane at a time, rows that allow only 8-byte
 // accesses (an odd number of complex vectors) four float2; a block with either in a pass takes this
 // instance. Its own instance, since its registers would cost the narrow rows a third of their warps in
@@ -391,7 +395,7 @@ template <typename T, bool C, bool WIDE>
 __global__ void __launch_bounds__(256, WIDE ? 0 : 5) k_node_update_multi(const NodeK* __restrict__ P,
                                                            const int64_t* __restrict__ node_off,
                                                            const int64_t* __restrict__ node_slot,
-                                                           const double* __restrict__ m, int64_t nh) {
+                                                           const float* __restrict__ minv_of, int64_t nh) {
   const NodeK p = P[blockIdx.y];
   constexpr int R = C ? 2 : 1;
   const int lane = threadIdx.x & 31;
@@ -405,9 +409,9 @@ __global__ void __launch_bounds__(256, WIDE ? 0 : 5) k_node_update_multi(const N
   const T* Rr = (const T*)p.R;
   const float* coef = p.coef;
   T* Y = (T*)p.Y;
-  const T alpha = (T)p.alpha, cs = (T)p.cshift, beta = (T)p.beta;
+  const T alpha = p.falpha, cs = p.fcshift, beta = p.fbeta;
   const bool has_z = Z != nullptr, has_k = Xk != nullptr, has_r = Rr != nullptr;
-  const bool has_m1 = p.beta != 0.0 && Xm1 != nullptr;
+  const bool has_m1 = __double_as_longlong(p.beta) << 1 != 0 && Xm1 != nullptr;
   const bool vec = sizeof(T) == 4 && W % 4 == 0 && ldy % 4 == 0 && ((uintptr_t)Y & 15) == 0 &&
                    (!has_z || ((uintptr_t)Z & 15) == 0) &&
                    (!has_k || (ldk % 4 == 0 && ((uintptr_t)Xk & 15) == 0)) &&
@@ -463,7 +467,7 @@ __global__ void __launch_bounds__(256, WIDE ? 0 : 5) k_node_update_multi(const N
       for (int u = 0; u < 2; ++u) {
         if (!ok[u] || !act) continue;
         const int64_t g = gg[u];
-        const T minv = (T)(1.0 / m[g]);
+        const T minv = minv_of[g];
         const float4 xk = has_k ? *reinterpret_cast<const float4*>((const float*)Xk + g * ldk + f)
                                 : make_float4(0.f, 0.f, 0.f, 0.f);
         float4 o;
@@ -493,7 +497,7 @@ __global__ void __launch_bounds__(256, WIDE ? 0 : 5) k_node_update_multi(const N
   for (int64_t g = warp0; g < nh; g += nwarps) {
     const int64_t s0 = node_off[g];
     const int ns = has_z ? (int)(node_off[g + 1] - s0) : 0;
-    const T minv = (T)(1.0 / m[g]);
+    const T minv = minv_of[g];
     if (WIDE && vec) {
       node_row<float4, 3, R>(p, Z, node_slot + s0, ns, g, W, ldk, ldm1, ldy, ldr, (float)minv, has_k, has_m1, has_r);
     } else if (WIDE && vec2) {
@@ -923,7 +927,7 @@ int batched_launch_degrees(oefe_ctx* c, const BatchPlan& P, bool cplx, const Mma
       wide = wide || W > 128 || W % 4 != 0;
     }
     auto node = [&](auto kern) {
-      OEFE_COUNTED kern<<<g1, 256, 0, c->bstream>>>(d_nd + (size_t)j * P.nk, c->d_node_off, c->d_node_slot, c->d_m, c->nh);
+      OEFE_COUNTED kern<<<g1, 256, 0, c->bstream>>>(d_nd + (size_t)j * P.nk, c->d_node_off, c->d_node_slot, c->d_minv, c->nh);
     };
     if (cplx) {
       if (wide) node(k_node_update_multi<float, true, true>);
@@ -1102,6 +1106,9 @@ int filter_batched_impl(oefe_ctx* c, int nk, void* const* X, const int* nv, cons
       nd.alpha = alpha;
       nd.cshift = cc;
       nd.beta = beta;
+      nd.falpha = (float)alpha;
+      nd.fcshift = (float)cc;
+      nd.fbeta = (float)beta;
       nd.R = nullptr;
       nd.coef = nullptr;
       nd.ldr = 0;

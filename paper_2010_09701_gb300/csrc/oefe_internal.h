@@ -120,6 +120,7 @@ struct oefe_ctx {
   std::vector<double> gll_x, gll_w;
   double* d_gll = nullptr;       // P nodes
   double* d_m = nullptr;         // nh lumped masses
+  float* d_minv = nullptr;       // their reciprocals, for the FP32 filter
   int* d_cell_nodes = nullptr;   // ncells * nloc
   double* d_cellbox = nullptr;   // ncells * 6 (lo xyz, h xyz)
   std::vector<int> cell_nodes;   // host copy

@@ -173,6 +173,9 @@ int setup_mesh(oefe_ctx* c, double a, const int ncell[3], const double* xb, int 
         }
   }
   OEFE_TRY(upload(c, &c->d_m, m));
+  std::vector<float> mi(m.size());
+  for (size_t i = 0; i < m.size(); ++i) mi[i] = (float)(1.0 / m[i]);
+  OEFE_TRY(upload(c, &c->d_minv, mi));
   OEFE_TRY(upload(c, &c->d_cell_nodes, c->cell_nodes));
   OEFE_TRY(upload(c, &c->d_cellbox, box));
   OEFE_TRY(upload(c, &c->d_gll, c->gll_x));
