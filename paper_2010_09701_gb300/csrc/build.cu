@@ -1425,6 +1425,7 @@ static int run_cell_kernel(oefe_ctx* c, KData& K, int mode, const double* veff, 
 int setup_kpoints(oefe_ctx* c, int nk, const double* k, const double* w) {
   if (!c->has_quad) { c->err = "kpoints: call oefe_quadrature first"; return OEFE_ERR_STATE; }
   if (nk < 1 || nk > 4096 || !k || !w) { c->err = "kpoints: need 1 <= nk <= 4096, k, w"; return OEFE_ERR_ARG; }
+  release_batch_graphs(c);
   for (auto& K : c->kd) {
     dev_free(K.gamma); dev_free(K.Moo); dev_free(K.Mooinv); dev_free(K.H64); dev_free(K.H32); dev_free(K.Hbf); dev_free(K.Hp);
     dev_free(K.E0); dev_free(K.NO); dev_free(K.NOp);
@@ -1557,6 +1558,7 @@ int build_hamiltonian(oefe_ctx* c, const double* veff, int store) {
     if (st == OEFE_OK) st = keep((void**)&K.Hp, store & OEFE_STORE_F64PAIR, n64 * sb);
     const int parts = (store & OEFE_STORE_BF16X6) ? 3 : (store & OEFE_STORE_BF16X3) ? 2 : 0;
     if (parts != K.bf_parts) {   // a different split: a new buffer
+      release_batch_graphs(c);
       dev_free(K.Hbf);
       K.Hbf = nullptr;
     }

@@ -1532,7 +1532,10 @@ int filter_autotune(oefe_ctx* c, int nk, void* const* X, const int* nv, const in
   return OEFE_OK;
 }
 
+// The captured launches hold the addresses of the context's tables and stored matrices, which their key does
+// not name: whatever replaces one of them (mesh, enrichment, k-points, another split) calls this first.
 void release_batch_graphs(oefe_ctx* c) {
+  if (!c->bgraphs.empty() && c->bstream) cudaStreamSynchronize(c->bstream);
   for (auto& g : c->bgraphs) {
     if (g.exec) cudaGraphExecDestroy(g.exec);
     dev_free(g.params);

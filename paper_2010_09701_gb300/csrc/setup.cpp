@@ -172,6 +172,7 @@ int setup_mesh(oefe_ctx* c, double a, const int ncell[3], const double* xb, int 
           m[g] += c->gll_w[i] * c->gll_w[j] * c->gll_w[k] * vol8;
         }
   }
+  release_batch_graphs(c);
   OEFE_TRY(upload(c, &c->d_m, m));
   std::vector<float> mi(m.size());
   for (size_t i = 0; i < m.size(); ++i) mi[i] = (float)(1.0 / m[i]);
@@ -303,6 +304,7 @@ int setup_enrichment(oefe_ctx* c, int natoms, const double* pos, int nfun, const
     Rv.assign(R, R + (size_t)natoms * nfun * ngrid);
     dRv.assign(dR, dR + (size_t)natoms * nfun * ngrid);
   }
+  release_batch_graphs(c);
   OEFE_TRY(upload(c, &c->d_R, Rv));
   OEFE_TRY(upload(c, &c->d_dR, dRv));
   OEFE_TRY(upload(c, &c->d_pos, c->pos));
