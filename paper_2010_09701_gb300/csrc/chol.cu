@@ -68,7 +68,10 @@ __global__ void __launch_bounds__(CB * CB) k_chol_step(S* __restrict__ A, S* __r
                                                        int p, int* info) {
   __shared__ S li[CB][CB + 1], lk[CB][CB + 1], lp[CB][CB + 1];
   __shared__ double iv[CB];
-  if (*info) return;
+  // only a failure of an earlier launch counts (its pivot lies in the blocks up to p): the diagonal block of this
+  // launch may report one while other CTAs start, and a CTA must take one decision
+  const int failed = *(volatile int*)info;
+  if (failed && failed <= (p + 1) * CB) return;
   const int r = threadIdx.x / CB, c = threadIdx.x % CB;
   // blockIdx.x enumerates the pairs (i, k), i >= k, of the trailing blocks row by row
   int bi = 0, t = blockIdx.x;
