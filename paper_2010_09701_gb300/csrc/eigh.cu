@@ -12,7 +12,10 @@
 namespace {
 
 constexpr int JT = 1024;
-constexpr int MAXPAIRS = 512;   // n <= 1024
+constexpr int MAXN = 1024;
+// one CTA takes matrices up to this size: A and V in its shared memory (204800 bytes) beside the rotations and
+// the reduction (9792)
+constexpr int CTA_N = 80;
 
 __device__ inline double block_sum(double v, double* red) {
   const int tid = threadIdx.x;
@@ -67,9 +70,9 @@ __global__ void __launch_bounds__(JT) k_jacobi(cd* Ag, cd* Vg, int n, int max_sw
     __syncthreads();
   }
   __shared__ double red[JT];
-  __shared__ double cs_[MAXPAIRS], sn_[MAXPAIRS];
-  __shared__ cd u_[MAXPAIRS];
-  __shared__ int p_[MAXPAIRS], q_[MAXPAIRS];
+  __shared__ double cs_[CTA_N / 2], sn_[CTA_N / 2];
+  __shared__ cd u_[CTA_N / 2];
+  __shared__ int p_[CTA_N / 2], q_[CTA_N / 2];
   const int tid = threadIdx.x;
   const int m = n + (n & 1);  // even number of players; player n is a bye when n is odd
   const int np = m / 2;
@@ -470,7 +473,7 @@ __global__ void k_from_cd(const cd* B, S* A, int n2) {
 // Returns OEFE_ERR_CHOLESKY if M is not positive definite.
 template <typename S>
 int gpu_geneig(oefe_ctx* c, const S* H, const S* M, int n, double* eps_host, S* U) {
-  if (n > 2 * MAXPAIRS) { c->err = "eigensolver: n too large"; return OEFE_ERR_ARG; }
+  if (n > MAXN) { c->err = "eigensolver: n too large"; return OEFE_ERR_ARG; }
   const size_t nn = (size_t)n * n;
   auto a256 = [](size_t x) { return ((x + 255) / 256) * 256; };
   const size_t nb = a256(nn * sizeof(cd)), eb = a256((size_t)n * sizeof(double)), cb = a256(chol_scratch(n));
@@ -523,7 +526,7 @@ int gpu_geneig(oefe_ctx* c, const S* H, const S* M, int n, double* eps_host, S* 
       OEFE_CUDA_TRY(c, cudaMemcpyAsync(&fail, bar.fail, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
       return OEFE_OK;
     };
-    if (c->f64_products == OEFE_F64_PAIRS && jsm <= 200 * 1024) {
+    if (c->f64_products == OEFE_F64_PAIRS && n <= CTA_N) {
       // the sweeps down to about the pair precision on the FP32 pipe, the rest (usually none: Jacobi
       // converges quadratically) in FP64; the result carries the pair arithmetic's backward error,
       // about 2^-48 ||A||
