@@ -1338,8 +1338,8 @@ namespace {
 // buffers; each group keeps its own captured graph. A pass of every column streams the cell matrices
 // once (the tiles of one cell's vector blocks are neighbours in the launch order, so all but the first
 // read them from L2), so every column goes in one pass when its buffers take at most 1 / FILTER_WS_SHARE
-// of the device's memory, else groups of FILTER_CHUNK: 360 real columns on the 16^3 supercell (12 GB)
-// take one pass instead of three, on the 32^3 one (95 GB) three.
+// of the device's memory and no more than they leave free, else groups of FILTER_CHUNK: 360 real columns on
+// the 16^3 supercell (12 GB) take one pass instead of three, on the 32^3 one (95 GB) three.
 constexpr int FILTER_CHUNK = 128;
 constexpr int FILTER_WS_SHARE = 8;
 
@@ -1350,7 +1350,8 @@ int filter_groups(const oefe_ctx* c, int nk, const int* nv, int vmax, int dtype)
   const double per = (double)c->ncells * c->npad * es_low + n * (3.0 * es_low + (dtype_fp64(dtype) ? 2.0 * es : 0.0));
   double bytes = 0;
   for (int k = 0; k < nk; ++k) bytes += (double)nv[k] * per;
-  return bytes * FILTER_WS_SHARE <= (double)c->dev_bytes ? 1 : most;
+  if (bytes * FILTER_WS_SHARE > (double)c->dev_bytes) return most;
+  return bytes <= (double)c->ws_bytes || bytes <= (double)ws_room(c) ? 1 : most;
 }
 
 int filter_batched_groups(oefe_ctx* c, int nk, void* const* X, const int* nv, const int* ld, int dtype, int degree,
@@ -1361,10 +1362,16 @@ int filter_batched_groups(oefe_ctx* c, int nk, void* const* X, const int* nv, co
     ok = nv[k] >= 1;
     vmax = std::max(vmax, ok ? nv[k] : 0);
   }
-  const int Q = ok && dtype >= 0 && dtype <= 3 ? filter_groups(c, nk, nv, vmax, dtype) : 1;
-  for (int k = 0; ok && k < nk; ++k) ok = nv[k] >= Q;
-  if (!ok || Q <= 1 || dtype < 0 || dtype > 3)   // one pass (the call checks its arguments itself)
-    return filter_batched_impl(c, nk, X, nv, ld, dtype, degree, a, b, a0, theta, flags);
+  int Q = ok && dtype >= 0 && dtype <= 3 ? filter_groups(c, nk, nv, vmax, dtype) : 1;
+  const int most = (vmax + FILTER_CHUNK - 1) / FILTER_CHUNK;
+  bool split = ok && most > 1 && dtype >= 0 && dtype <= 3;   // the columns can be grouped
+  for (int k = 0; split && k < nk; ++k) split = nv[k] >= most;
+  if (!split || Q <= 1) {   // one pass (the call checks its arguments itself)
+    const int st = filter_batched_impl(c, nk, X, nv, ld, dtype, degree, a, b, a0, theta, flags);
+    // (beyond degree 1, its allocations come before it touches the vectors)
+    if (st != OEFE_ERR_OOM || !split || degree < 2) return st;
+    Q = most;
+  }
   const size_t es = dtype_bytes(dtype);
   std::vector<size_t> toff(nk + 1, 0);
   for (int k = 0; k < nk; ++k) toff[k + 1] = toff[k] + nv[k];

@@ -223,6 +223,8 @@ cudaEvent_t timing_event(oefe_ctx* c);
 
 // ------------------------------------------------------------------ internals
 int ensure_ws(oefe_ctx* c, size_t bytes);
+// bytes that the workspace may take and leave the caller as much: what it holds, or half of that and the free memory
+size_t ws_room(const oefe_ctx* c);
 int ensure_ws2(oefe_ctx* c, size_t bytes);
 int dev_alloc(oefe_ctx* c, void** p, size_t bytes);
 void dev_free(void* p);

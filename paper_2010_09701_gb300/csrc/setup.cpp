@@ -105,6 +105,15 @@ int ensure_ws(oefe_ctx* c, size_t bytes) {
   return OEFE_OK;
 }
 
+size_t ws_room(const oefe_ctx* c) {
+  size_t fr = 0, tot = 0;
+  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+    cudaGetLastError();
+    fr = 0;
+  }
+  return std::max(c->ws_bytes, (fr + c->ws_bytes) / 2);
+}
+
 int ensure_ws2(oefe_ctx* c, size_t bytes) {
   if (bytes <= c->ws2_bytes) return OEFE_OK;
   cudaStreamSynchronize(c->stream);
