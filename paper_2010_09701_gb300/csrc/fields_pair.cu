@@ -354,25 +354,41 @@ int fields_pair(oefe_ctx* c, KData& K, const void* X, int nv, int ld, bool cplx,
   const int P = c->P, R = cplx ? 2 : 1;
   if (P < 4 || P > 7 || c->nq_cell != P || c->nq_enr != P + 2 || R * c->ne_max > ZMAXK) return OEFE_OK;
   const int ncr = nv * R, vblocks = (ncr + ZN - 1) / ZN, ncp = (ncr + 1) / 2;
-  // batches of leaves whose workspace stays below a 32nd of the device
   const int nl_all = (int)c->leaves.size();
-  const double per_point = (double)ncp * sizeof(float4);
-  size_t ws = 0;
-  std::vector<int> cut{0};
-  {
+  const size_t per_point = (size_t)ncp * sizeof(float4);
+  std::vector<int> cut{0, nl_all};
+  // the leaves in batches whose workspace takes at most cap bytes (or one leaf's): the workspace
+  auto batches = [&](size_t cap) -> size_t {
+    size_t ws = 0;
     int64_t q0 = 0;
+    cut.assign(1, 0);
     for (int i = 0; i < nl_all; ++i) {
       const int64_t q1 = i + 1 < nl_all ? c->leaves[i + 1].q0 : c->nq;
-      if ((double)(q1 - q0) * per_point * 32 > (double)c->dev_bytes && i > cut.back()) {
+      if ((size_t)(q1 - q0) * per_point > cap && i > cut.back()) {
         cut.push_back(i);
         q0 = c->leaves[i].q0;
       }
-      ws = std::max(ws, (size_t)((double)(q1 - q0) * per_point));
+      ws = std::max(ws, (size_t)(q1 - q0) * per_point);
     }
     cut.push_back(nl_all);
-  }
+    return ws;
+  };
   const bool enr = c->nO > 0 && c->ne_max > 0;
-  if (enr) OEFE_TRY(ensure_ws(c, ws + 256));
+  if (enr) {
+    // a 32nd of the device at most, and no more than that leaves free; smaller batches when the allocation fails.
+    // Batches of less than half a leaf per SM would leave this path slower than the general kernel, which
+    // needs no workspace (2.6 times as long on a full GPU)
+    size_t ws = batches(std::max(c->dev_bytes / 32, (size_t)64 << 20));
+    if (ws + 256 > c->ws_bytes) ws = batches(std::min(ws, ws_room(c)));
+    int st = OEFE_ERR_OOM;
+    while ((int)cut.size() == 2 || ((long long)cut.size() - 1) * (c->num_sms / 2) <= nl_all) {
+      st = ensure_ws(c, ws + 256);
+      if (st != OEFE_ERR_OOM || (int)cut.size() > nl_all) break;
+      ws = batches(ws / 2);
+    }
+    if (st == OEFE_ERR_OOM) return OEFE_OK;
+    OEFE_TRY(st);
+  }
   const int n1m = std::max(c->nq_cell, c->nq_enr);
   for (size_t bi = 0; bi + 1 < cut.size(); ++bi) {
     const int l0 = cut[bi], nl = cut[bi + 1] - l0;

@@ -7,7 +7,7 @@ import pytest
 import torch
 
 import workloads as W
-from gpu_cases import paired, to_gpu
+from gpu_cases import paired, rel, to_gpu
 from oracle import solver
 
 pytestmark = pytest.mark.gpu
@@ -21,9 +21,9 @@ def device_memory_left(nbytes):
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     held = []
-    for block in (1024 * MB, 32 * MB, 2 * MB):
-        while torch.cuda.mem_get_info()[0] >= nbytes + block:
-            held.append(torch.empty(block, dtype=torch.uint8, device="cuda"))
+    while torch.cuda.mem_get_info()[0] >= nbytes + 2048 * MB:
+        held.append(torch.empty(1024 * MB, dtype=torch.uint8, device="cuda"))
+    held.append(torch.empty(torch.cuda.mem_get_info()[0] - nbytes - 2 * MB, dtype=torch.uint8, device="cuda"))
     try:
         yield
     finally:
@@ -73,3 +73,43 @@ def test_batched_filter_takes_column_groups():
     with device_memory_left(64 * MB):
         groups = both()
     assert groups == [3 * n for n in one]
+
+
+@pytest.mark.parametrize("k", [(0.0, 0.0, 0.0), (0.25, -0.4, 0.1)])
+def test_fields_in_batches_of_leaves(k):
+    # pair mode, 328 leaves of 4^3 and 6^3 points; room for all of them, for a part, for too few to be worth it
+    # (the general kernel). Tolerance of the fields in pairs elsewhere in this suite.
+    from paper_2010_09701_gb300 import F64_PAIRS, STORE_F64, STORE_F64PAIR, launch_count
+    nv = 67 if any(k) else 131
+    prs, ctx, V, Vd = paired(ks=[k], n=6, a=12.0, p=3, quad=(4, 6, 1), store=STORE_F64 | STORE_F64PAIR)
+    pr = prs[0]
+    ctx.set_f64_products(F64_PAIRS)
+    X = W.random_vectors(pr.n, nv, complex_=pr.complex, seed=95)
+    occ = np.linspace(2.0, 0.0, nv)
+    Xd = to_gpu(X)
+    rho = torch.empty(pr.quad.nq, dtype=torch.float64, device="cuda")
+    g, g2 = torch.empty_like(rho), torch.empty_like(rho)
+    rho_o, g_o = solver.density([pr], [X], [occ]), solver.band_trace_grad_V(pr, X)
+    ncp = nv if pr.complex else (nv + 1) // 2
+    full = pr.quad.nq * ncp * 16
+
+    def fields():
+        n0 = launch_count()
+        ctx.density_grad([Xd], [occ], rho, 0, g)
+        n1 = launch_count()
+        ctx.band_trace_grad(0, Xd, g2)
+        n2 = launch_count()
+        for out, ref in ((rho, rho_o), (g, g_o), (g2, g_o)):
+            assert rel(out.cpu().numpy(), ref) < 3.2e-12
+        return n1 - n0, n2 - n1
+
+    fields()                           # (the first call forms the pair copy of the enrichment table)
+    assert fields() == (3, 3)          # the enrichment part, the two rules
+    ctx.release_workspace()
+    with device_memory_left(full):     # half of it: two or three batches
+        assert fields() in ((6, 6), (9, 9))
+    ctx.release_workspace()
+    with device_memory_left(full // 8):
+        assert fields()[1] == 1        # the general kernel
+    ctx.release_workspace()
+    assert fields() == (3, 3)
