@@ -64,9 +64,9 @@ __global__ void __launch_bounds__(FZ, 1) k_fields_oz(const FieldOzArgs A) {
   for (long long job = blockIdx.x; job < total && !s_fail; job += gridDim.x) {
     const Leaf L = A.leaves[A.l0 + job / A.mtiles];
     const int n3 = L.n1 * L.n1 * L.n1, p0 = (int)(job % A.mtiles) * 128;
-    if (p0 >= n3) continue;
-    const int nr = min(128, n3 - p0);
     const int o0 = A.act_off[L.cell], ne = A.act_off[L.cell + 1] - o0;
+    if (p0 >= n3 || ne == 0) continue;   // (k_fields_cc does not read the part of a leaf without active functions)
+    const int nr = min(128, n3 - p0);
     const bool aok = ar < nr;
     const double* no = A.NO + R * ((size_t)L.q0 * A.ne_max + p0 + ar);
     const size_t cs = (size_t)R * n3;                  // reals between columns of the table
