@@ -52,3 +52,9 @@ def _check(name, nvs):
 @pytest.mark.parametrize("name", ["none_real", "none_complex"])
 def test_cells_without_functions(name):
     _check(name, (1, 33, 70))
+
+
+@pytest.mark.parametrize("name", ["many_complex", "many_real"])
+def test_more_functions_than_one_pass(name):
+    # the operand halves are used again and the table's digits are cut anew for every column block
+    _check(name, (1, 33, 131))
