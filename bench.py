@@ -47,10 +47,12 @@ TRAFFIC_TENSOR = {   # bf16 parts of the split -> DRAM bytes per (k, cell, 64-ve
     2: {"bytes_per_tile": (2.044714e9 + 0.008223e9) / 1728, "source": "profiles/k_cell_mma_tma_c3mid_12cube_p6.md"},
     3: {"bytes_per_tile": (3.064588e9 + 0.008374e9) / 1728, "source": "profiles/k_cell_mma_tma_c3mid_12cube_p6.md"},
 }
-TRAFFIC_FP64 = None   # {"bytes_per_cell", "source"} from a capture of the current FP64 product kernels
-# the FP64-class products in pair mode: DRAM bytes of the single-leaf cells' kernels per launch of 64 columns and
-# cell, {"sf_bytes_per_cell", "source"} from a capture of the current kernels
-TRAFFIC_PAIR = None
+# the FP64-class products in pair mode, by real and complex data: DRAM bytes of the single-leaf cells' kernels per
+# launch of 64 columns and cell; the refined cells' dense product is not in it
+TRAFFIC_PAIR = {
+    False: {"sf_bytes_per_cell": (0.517e9 + 0.836e9 + 2.61e9 + 0.732e9) / 3600, "where": "62-atom cell, 16^3 mesh"},
+    True: {"sf_bytes_per_cell": (0.115e9 + 0.176e9 + 0.472e9 + 0.146e9) / 448, "where": "8-atom cell, 8^3 mesh"},
+}
 
 
 def is_complex(w):
@@ -574,11 +576,10 @@ def run_ours(args, rank, world):
         n_dense = nucleus_cells(w)
         n_sf = len(naug) - n_dense
         traffic = None
-        if pairs and TRAFFIC_PAIR and not cplx:
-            traffic = {"bytes": TRAFFIC_PAIR["sf_bytes_per_cell"] * n_sf, "source": TRAFFIC_PAIR["source"]}
-        elif not pairs and TRAFFIC_FP64:
-            traffic = {"bytes": TRAFFIC_FP64["bytes_per_cell"] * len(naug),
-                       "source": TRAFFIC_FP64["source"] + " (scaled by cells)"}
+        if pairs:
+            traffic = {"bytes": TRAFFIC_PAIR[cplx]["sf_bytes_per_cell"] * n_sf,
+                       "source": ("profiles/pair_products_dram_bytes_p6.md: k_sf_cc + k_sf_strips per single-leaf cell (%s), "
+                                  "scaled by the single-leaf cells" % TRAFFIC_PAIR[cplx]["where"])}
         if pairs:
             # the refined cells (dense FP64) take a few percent of the launch; the peak is that of
             # the pair arithmetic on the FP32 pipe
