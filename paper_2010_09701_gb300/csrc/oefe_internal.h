@@ -249,6 +249,10 @@ int rotate_ozaki(oefe_ctx* c, S* X, int ldx, int64_t n, int nv, const S* C, bool
 // the same for any nv, the digits cut inside the MMA kernels (ozaki_wide.cu)
 template <typename S>
 int gram_ozaki_wide(oefe_ctx* c, const S* X, int ldx, const S* W, int ldw, int64_t n, int nv, S* out, bool herm);
+// the buffer of the digit kernels' planes and partial sums, grown; the end of a call of theirs: wait and read
+// their error word (d_status + 2)
+int grow_ozpart(oefe_ctx* c, size_t need);
+int oz_finish(oefe_ctx* c, const char* what);
 // Gram matrices and rotations of wider blocks from eight digits (oz8_wide.cu)
 template <typename S>
 int gram_oz8(oefe_ctx* c, const S* X, int ldx, const S* W, int ldw, int64_t n, int nv, S* out, bool herm);

@@ -331,30 +331,6 @@ __global__ void __launch_bounds__(WT, 1) k_rot_oz8(const WRotArgs A) {
   oz_end(C, H, &s_fail, A.err);
 }
 
-int grow_ozpart(oefe_ctx* c, size_t need) {
-  if (c->ozpart_bytes >= need) return OEFE_OK;
-  cudaStreamSynchronize(c->stream);
-  dev_free(c->d_ozpart);
-  c->d_ozpart = nullptr;
-  c->ozpart_bytes = 0;
-  OEFE_TRY(dev_alloc(c, &c->d_ozpart, need));
-  c->ozpart_bytes = need;
-  return OEFE_OK;
-}
-
-int finish_wide(oefe_ctx* c, const char* what) {
-  OEFE_CUDA_TRY(c, cudaGetLastError());
-  int flag = 0;
-  OEFE_CUDA_TRY(c, cudaMemcpyAsync(&flag, c->d_status + 2, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  if (flag) {
-    cudaMemsetAsync(c->d_status + 2, 0, sizeof(int), c->stream);
-    c->err = std::string(what) + ": a tensor-core wait timed out";
-    return OEFE_ERR_TIMEOUT;
-  }
-  return OEFE_OK;
-}
-
 size_t a256(size_t x) { return ((x + 255) / 256) * 256; }
 
 }  // namespace
@@ -402,7 +378,7 @@ int gram_oz8(oefe_ctx* c, const S* X, int ldx, const S* W, int ldw, int64_t n, i
   OEFE_COUNTED k_oz_col_exps<<<(unsigned)A.chunks, 256, 0, c->stream>>>(A.W, A.ldw, n, nvr, crows, ew);
   OEFE_COUNTED k_gram_oz8<<<dim3(used, ntile), WT, WSMEM, c->stream>>>(A);
   OEFE_COUNTED k_gram_oz8_reduce<S><<<(nv * nv + 255) / 256, 256, 0, c->stream>>>(A.part, used, nI, nJ, nv, herm, out);
-  return finish_wide(c, "gram");
+  return oz_finish(c, "gram");
 }
 
 // X[0:n] <- X G (G = C, or C^+ of a lower triangular C when herm) on the tensor cores
@@ -430,7 +406,7 @@ int rotate_oz8(oefe_ctx* c, S* X, int ldx, int64_t n, int nv, const S* C, bool h
   OEFE_COUNTED k_oz_col_exps<<<gch, 256, 0, c->stream>>>(A.G, A.nvr, A.nvr, A.nvr, ZMAXK, (int*)(base + gb));
   OEFE_CUDA_TRY(c, cudaFuncSetAttribute(k_rot_oz8, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WSMEM));
   OEFE_COUNTED k_rot_oz8<<<grid, WT, WSMEM, c->stream>>>(A);
-  return finish_wide(c, "rotate");
+  return oz_finish(c, "rotate");
 }
 
 template int gram_oz8<double>(oefe_ctx*, const double*, int, const double*, int, int64_t, int, double*, bool);

@@ -554,6 +554,30 @@ __global__ void k_gram_oz_reduce(const double* part, int nbx, int nv, S* out) {
 
 }  // namespace
 
+int grow_ozpart(oefe_ctx* c, size_t need) {
+  if (c->ozpart_bytes >= need) return OEFE_OK;
+  cudaStreamSynchronize(c->stream);
+  dev_free(c->d_ozpart);
+  c->d_ozpart = nullptr;
+  c->ozpart_bytes = 0;
+  OEFE_TRY(dev_alloc(c, &c->d_ozpart, need));
+  c->ozpart_bytes = need;
+  return OEFE_OK;
+}
+
+int oz_finish(oefe_ctx* c, const char* what) {
+  OEFE_CUDA_TRY(c, cudaGetLastError());
+  int flag = 0;
+  OEFE_CUDA_TRY(c, cudaMemcpyAsync(&flag, c->d_status + 2, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  if (flag) {
+    cudaMemsetAsync(c->d_status + 2, 0, sizeof(int), c->stream);
+    c->err = std::string(what) + ": a tensor-core wait timed out";
+    return OEFE_ERR_TIMEOUT;
+  }
+  return OEFE_OK;
+}
+
 // out = X^+ W (nv x nv) on the tensor cores; *done = false when the shape is not covered (nv > 64)
 template <typename S>
 int gram_ozaki(oefe_ctx* c, const S* X, int ldx, const S* W, int ldw, int64_t n, int nv, S* out, bool* done) {
@@ -567,14 +591,7 @@ int gram_ozaki(oefe_ctx* c, const S* X, int ldx, const S* W, int ldw, int64_t n,
   const size_t pl_bytes = a256((size_t)passes * PASS_BYTES), ex_bytes = a256((size_t)passes * 128 * sizeof(int));
   const size_t pt_bytes = a256((size_t)halves * nbx * 128 * OZ_N * sizeof(double));
   const size_t need = 2 * pl_bytes + 2 * ex_bytes + pt_bytes;
-  if (c->ozpart_bytes < need) {
-    cudaStreamSynchronize(c->stream);
-    dev_free(c->d_ozpart);
-    c->d_ozpart = nullptr;
-    c->ozpart_bytes = 0;
-    OEFE_TRY(dev_alloc(c, &c->d_ozpart, need));
-    c->ozpart_bytes = need;
-  }
+  OEFE_TRY(grow_ozpart(c, need));
   unsigned char* base = (unsigned char*)c->d_ozpart;
   unsigned char* pa = base;
   unsigned char* pbp = base + pl_bytes;
@@ -602,15 +619,7 @@ int gram_ozaki(oefe_ctx* c, const S* X, int ldx, const S* W, int ldw, int64_t n,
   dim3 grid(nbx, halves);
   OEFE_COUNTED k_gram_oz<<<grid, OZ_T, OZ_SMEM, c->stream>>>(A);
   OEFE_COUNTED k_gram_oz_reduce<S><<<(nv * nv + 255) / 256, 256, 0, c->stream>>>(part, nbx, nv, out);
-  OEFE_CUDA_TRY(c, cudaGetLastError());
-  int flag = 0;
-  OEFE_CUDA_TRY(c, cudaMemcpyAsync(&flag, c->d_status + 2, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  if (flag) {
-    cudaMemsetAsync(c->d_status + 2, 0, sizeof(int), c->stream);
-    c->err = "gram: a tensor-core wait timed out";
-    return OEFE_ERR_TIMEOUT;
-  }
+  OEFE_TRY(oz_finish(c, "gram"));
   *done = true;
   return OEFE_OK;
 }
@@ -630,14 +639,7 @@ int rotate_ozaki(oefe_ctx* c, S* X, int ldx, int64_t n, int nv, const S* C, bool
   const size_t pa_bytes = a256((size_t)tiles * 2 * PASS_BYTES), ea_bytes = a256((size_t)tiles * 128 * sizeof(int));
   const size_t pb_bytes = a256((size_t)4 * OZ_S * BH), eb_bytes = 256 + 128 * sizeof(int);
   const size_t need = pa_bytes + ea_bytes + pb_bytes + eb_bytes;
-  if (c->ozpart_bytes < need) {
-    cudaStreamSynchronize(c->stream);
-    dev_free(c->d_ozpart);
-    c->d_ozpart = nullptr;
-    c->ozpart_bytes = 0;
-    OEFE_TRY(dev_alloc(c, &c->d_ozpart, need));
-    c->ozpart_bytes = need;
-  }
+  OEFE_TRY(grow_ozpart(c, need));
   unsigned char* base = (unsigned char*)c->d_ozpart;
   unsigned char* pa = base;
   int* ea = (int*)(base + pa_bytes);
@@ -663,15 +665,7 @@ int rotate_ozaki(oefe_ctx* c, S* X, int ldx, int64_t n, int nv, const S* C, bool
   OEFE_CUDA_TRY(c, cudaFuncSetAttribute(k_rot_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM));
   const int grid = (int)std::min<long long>(tiles, c->num_sms);
   OEFE_COUNTED k_rot_oz<<<grid, OZ_T, OZ_SMEM, c->stream>>>(A);
-  OEFE_CUDA_TRY(c, cudaGetLastError());
-  int flag = 0;
-  OEFE_CUDA_TRY(c, cudaMemcpyAsync(&flag, c->d_status + 2, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  if (flag) {
-    cudaMemsetAsync(c->d_status + 2, 0, sizeof(int), c->stream);
-    c->err = "rotate: a tensor-core wait timed out";
-    return OEFE_ERR_TIMEOUT;
-  }
+  OEFE_TRY(oz_finish(c, "rotate"));
   *done = true;
   return OEFE_OK;
 }

@@ -250,30 +250,6 @@ __global__ void k_gram_wide_reduce(const double* part, int nbx, int nI, int nJ, 
   else out[t] = D(i, j);
 }
 
-int grow_ozpart(oefe_ctx* c, size_t need) {
-  if (c->ozpart_bytes >= need) return OEFE_OK;
-  cudaStreamSynchronize(c->stream);
-  dev_free(c->d_ozpart);
-  c->d_ozpart = nullptr;
-  c->ozpart_bytes = 0;
-  OEFE_TRY(dev_alloc(c, &c->d_ozpart, need));
-  c->ozpart_bytes = need;
-  return OEFE_OK;
-}
-
-int finish_wide(oefe_ctx* c, const char* what) {
-  OEFE_CUDA_TRY(c, cudaGetLastError());
-  int flag = 0;
-  OEFE_CUDA_TRY(c, cudaMemcpyAsync(&flag, c->d_status + 2, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  if (flag) {
-    cudaMemsetAsync(c->d_status + 2, 0, sizeof(int), c->stream);
-    c->err = std::string(what) + ": a tensor-core wait timed out";
-    return OEFE_ERR_TIMEOUT;
-  }
-  return OEFE_OK;
-}
-
 }  // namespace
 
 // out = X^+ W (nv x nv) on the tensor cores, any nv; herm: the result is known to be Hermitian
@@ -313,7 +289,7 @@ int gram_ozaki_wide(oefe_ctx* c, const S* X, int ldx, const S* W, int ldw, int64
   dim3 grid(nbx, ntile);
   OEFE_COUNTED k_gram_wide<<<grid, WT, WSMEM, c->stream>>>(A);
   OEFE_COUNTED k_gram_wide_reduce<S><<<(nv * nv + 255) / 256, 256, 0, c->stream>>>(A.part, nbx, nI, nJ, nv, upper, out);
-  return finish_wide(c, "gram");
+  return oz_finish(c, "gram");
 }
 
 template int gram_ozaki_wide<double>(oefe_ctx*, const double*, int, const double*, int, int64_t, int, double*, bool);
