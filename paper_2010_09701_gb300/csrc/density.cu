@@ -530,7 +530,7 @@ int run_fields(oefe_ctx* c, KData& K, const void* X, int nv, int ld, int dtype, 
 
 // end of a fields call: wait, and in pair mode read the tensor-core kernels' error word
 int finish_fields(oefe_ctx* c) {
-  if (c->f64_products == OEFE_F64_PAIRS) return oz_status(c, "fields");
+  if (c->f64_products == OEFE_F64_PAIRS) return oz_finish(c, "fields");
   OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   return OEFE_OK;
 }

@@ -411,7 +411,7 @@ int fields_pair(oefe_ctx* c, KData& K, const void* X, int nv, int ld, bool cplx,
       A.q0 = q0;
       A.U = (float4*)c->ws;
       A.ncp = ncp;
-      A.err = c->d_status;
+      A.err = c->d_status + 2;
       const int grid = (int)std::min<long long>((long long)nl * A.mtiles, c->num_sms);
       auto go = [&](auto kern) -> int {
         OEFE_CUDA_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM));
@@ -457,18 +457,5 @@ int fields_pair(oefe_ctx* c, KData& K, const void* X, int nv, int ld, bool cplx,
     OEFE_CUDA_TRY(c, cudaGetLastError());
   }
   *done = true;
-  return OEFE_OK;
-}
-
-// after a fields call: wait, and read the error word of the tensor-core kernels
-int oz_status(oefe_ctx* c, const char* what) {
-  int flag = 0;
-  OEFE_CUDA_TRY(c, cudaMemcpyAsync(&flag, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  OEFE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  if (flag) {
-    cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
-    c->err = std::string(what) + ": a tensor-core wait timed out";
-    return OEFE_ERR_TIMEOUT;
-  }
   return OEFE_OK;
 }

@@ -448,7 +448,7 @@ int nchunks_for(oefe_ctx* c, int nv) {
 template <typename S>
 int chol_inverse_t(oefe_ctx* c, S* A, int n, bool inverse, S* Y, int* info_host) {
   OEFE_TRY(ensure_ws2(c, 256));
-  int* d_info = c->d_status;
+  int* d_info = c->d_status + 3;   // (a failure is no timeout: word 0 is the waits')
   OEFE_COUNTED k_chol<S><<<1, 1024, 0, c->stream>>>(A, n, d_info);
   OEFE_CUDA_TRY(c, cudaGetLastError());
   OEFE_CUDA_TRY(c, cudaMemcpyAsync(info_host, d_info, sizeof(int), cudaMemcpyDeviceToHost, c->stream));

@@ -177,7 +177,8 @@ struct oefe_ctx {
   size_t ws2_bytes = 0;
   void* d_ozpart = nullptr;             // partial sums of the tensor-core Gram matrices
   size_t ozpart_bytes = 0;
-  int* d_status = nullptr;        // device status word (Cholesky failures, timeouts)
+  // device status words: 0 timeouts of the cell products, 2 of the digit kernels, 3 the failing pivot of a Cholesky factor
+  int* d_status = nullptr;
 
   // optional event timing of the cell-product launches
   int timing = 0;  // dtype bit mask
@@ -337,8 +338,6 @@ int band_trace_grad(oefe_ctx* c, int ik, const void* X, int nv, int ld, int dtyp
 // the same sums in pair mode, enrichment part on the tensor cores (fields_pair.cu)
 int fields_pair(oefe_ctx* c, KData& K, const void* X, int nv, int ld, bool cplx, const double* occ, double* out,
                 bool density, double scale, double* out2, bool* done);
-// reads and clears the tensor-core kernels' error word (after a stream synchronization it joins)
-int oz_status(oefe_ctx* c, const char* what);
 // adjoint.cu
 int band_trace(oefe_ctx* c, int ik, const void* X, int nv, int ld, int dtype, double* e, void* HX);
 int band_trace_vjp(oefe_ctx* c, int ik, const void* X, int nv, int ld, int dtype, double alpha, double* gV, void* gX);

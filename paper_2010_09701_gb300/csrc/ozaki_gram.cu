@@ -614,7 +614,7 @@ int gram_ozaki(oefe_ctx* c, const S* X, int ldx, const S* W, int ldw, int64_t n,
   A.cplx = CPLX;
   A.nv = nv;
   A.part = part;
-  A.err = c->d_status + 2;   // its own word: the Cholesky kernels report through word 0
+  A.err = c->d_status + 2;
   OEFE_CUDA_TRY(c, cudaFuncSetAttribute(k_gram_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM));
   dim3 grid(nbx, halves);
   OEFE_COUNTED k_gram_oz<<<grid, OZ_T, OZ_SMEM, c->stream>>>(A);
