@@ -209,8 +209,11 @@ int oefe_chebyshev_filter(oefe_ctx_t ctx, int ik, void* X, int nv, int ld, int d
  * a private stream and replayed by later calls with the same arguments.
  * flags must contain OEFE_FILTER_BF16X3; with OEFE_FILTER_LAST_FP64 the
  * vectors are F64/C128 and the last degree runs per k in FP64, otherwise
- * they are F32/C64. X: host array of nk device pointers; nv, ld, a, b, a0:
- * host arrays of nk. The call returns after the filter has finished. */
+ * they are F32/C64. Blocks of more than 128 columns take one pass when its
+ * workspace is at most an eighth of the device memory and no more than it
+ * leaves free, else passes over groups of at most 128 columns. X: host array
+ * of nk device pointers; nv, ld, a, b, a0: host arrays of nk. The call returns
+ * after the filter has finished. */
 int oefe_filter_batched(oefe_ctx_t ctx, int nk, void* const* X, const int* nv, const int* ld, int dtype,
                         int degree, const double* a, const double* b, const double* a0, int flags);
 
@@ -401,7 +404,14 @@ int oefe_launch_count(int64_t* n);
  *     the projected matrices of wider blocks), and 8 balanced digits, about
  *     2^-53, for the Gram matrices of oefe_orthonormalize and every rotation of
  *     wider blocks; 8 digits also for the enrichment part of the fields where
- *     the rules have p + 1 and p + 3 points and p is 3 to 6.
+ *     the rules have p + 1 and p + 3 points and p is 3 to 6. The digits are
+ *     fixed point under a shared exponent, so values far below the largest that
+ *     share it keep fewer bits. Up to 64 vectors and in the projected matrices it
+ *     is shared by 64 rows of a column (Gram matrices) or a row of the block
+ *     (rotations); with 8 digits by at most 512 rows of a column (Gram
+ *     matrices), a row of the block and at most 512 rows of a column of the
+ *     small matrix (rotations), all functions at a point and a vector's
+ *     coefficients in a cell (fields; pairs hold 48 bits of every value).
  * Inputs and outputs stay FP64; Cholesky factors, triangular inverses and the
  * setup stay FP64. The operator must be built with OEFE_STORE_F64PAIR in pair
  * mode, else the products return OEFE_ERR_STATE; the build after the switch

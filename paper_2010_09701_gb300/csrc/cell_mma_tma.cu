@@ -116,9 +116,6 @@ __device__ __forceinline__ void decode_tile(const TmaArgs& A, long long t, int* 
   *vb = (int)(r % P.vblocks);
 }
 
-// MERGE (complex only): the real part of the cell matrix multiplies [Re X | Im X] in one N = 128
-// MMA instead of two N = 64 ones (fewer tensor instructions; which is faster depends on the split,
-// so the autotuner chooses)
 // the staged rows to a block of odd width or its tail, a vector per lane
 template <bool CPLX, int ER>
 __device__ __forceinline__ void store_ragged(const unsigned char* st, float* z, int nrows, int v, int nv) {
@@ -134,6 +131,9 @@ __device__ __forceinline__ void store_ragged(const unsigned char* st, float* z, 
   }
 }
 
+// MERGE (complex only): the real part of the cell matrix multiplies [Re X | Im X] in one N = 128
+// MMA instead of two N = 64 ones (fewer tensor instructions; which is faster depends on the split,
+// so the autotuner chooses)
 // NVT (real data only): vectors per tile, 64 or 128; with 128 a cell's matrix streams once for
 // twice the vectors (one N = 128 MMA per product, 128 tensor-memory columns per M tile).
 template <bool CPLX, int NPART, bool MERGE, int NVT = NBV>

@@ -4,13 +4,13 @@
 //   k_fields_oz  the enrichment part, a dense product of the stored N^O table with the enrichment
 //                coefficients, as an exact fixed-point product on the tensor cores (oz8_dev.cuh), into a
 //                workspace as FP32 pairs;
-//   k_fields_cc  the CFE part by sum factorization with register tiles (as sumfac_cc.cu), added to it,
+//   k_fields_cc  the CFE part by sum factorization with register tiles (as k_sf_cc, sumfac_pair.cu), added to it,
 //                squared, weighted and summed over the vectors without leaving registers.
 //
 // Bound: per leaf of 729 points and real vector the enrichment part was 28 k of 41 k pair multiply-adds,
 // on an FP32 pipe that the one-output-per-thread kernel (k_fields, density.cu) kept a third busy: 558 ms
 // for 360 vectors on the 62-atom cell at 16^3. On the tensor cores that part costs the cutting and combining
-// of its digits; the rest runs at the rate of sumfac_cc.cu. The workspace round trip (16 bytes per point
+// of its digits; the rest runs at the rate of k_sf_cc. The workspace round trip (16 bytes per point
 // and vector) is an eighth of the time saved.
 #include <algorithm>
 

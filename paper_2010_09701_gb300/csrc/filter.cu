@@ -615,8 +615,9 @@ struct Step {
 
 // Rows per CTA of the dense cell products: a CTA takes every row of its cell and vector block when
 // those blocks fill the GPU six times over (a last wave that is nearly empty then costs little), else
-// the rows are shared out (multiples of 16, one pass of the warps) until they do. Each row's sum is the same either way. The two-atom cell has 16 refined
-// cells, so 16 CTAs: 183 us a product of 20 real vectors, 757 us of 13 complex ones.
+// the rows are shared out in multiples of 8 until they do: a row a warp in k_cell_apply; k_cell_apply_z3 takes
+// two a warp, so at 8 rows half of its warps only gather. Each row's sum is the same either way. The two-atom
+// cell has 16 refined cells, so 16 CTAs: 183 us a product of 20 real vectors, 757 us of 13 complex ones.
 int dense_rows_per_cta(const oefe_ctx* c, long long blocks) {
   const int most = (c->npad + 7) / 8;
   const long long want = (6LL * c->num_sms + blocks - 1) / std::max(blocks, 1LL);
@@ -1338,8 +1339,11 @@ namespace {
 // buffers; each group keeps its own captured graph. A pass of every column streams the cell matrices
 // once (the tiles of one cell's vector blocks are neighbours in the launch order, so all but the first
 // read them from L2), so every column goes in one pass when its buffers take at most 1 / FILTER_WS_SHARE
-// of the device's memory and no more than they leave free, else groups of FILTER_CHUNK: 360 real columns on
-// the 16^3 supercell (12 GB) take one pass instead of three, on the 32^3 one (95 GB) three.
+// of the device's memory and no more than they leave free, else groups of FILTER_CHUNK. The share bounds the
+// memory, not the time, which is the lower in one pass at every width measured: ten BF16x3 degrees on the
+// 16^3 supercell take 57 ms in one pass and 62 in three groups at 360 real columns, 160 and 187 at 1080,
+// 298 and 563 at 2000 (16 groups, more than the graphs kept). 360 columns there need 12 GB; on the 32^3
+// supercell they would need 95 GB beside some 200 GB of operator and blocks, so three groups run.
 constexpr int FILTER_CHUNK = 128;
 constexpr int FILTER_WS_SHARE = 8;
 

@@ -1,8 +1,10 @@
 // Exact fixed-point products of FP64 operands on the tensor cores (the Ozaki scheme with bf16 digits):
-// shared by the cell products (cell_oz.cu) and the Gram matrices and rotations (ozaki_wide.cu).
+// shared by the Gram matrices and rotations of wide blocks (oz8_wide.cu) and the enrichment part of the fields
+// (fields_pair.cu).
 //
 // A value is cut into 8 balanced digits of 7 bits (each in [-64, 64), exact in bf16) under one exponent
-// per operand row: 54 bits of the row's largest value, more than an FP64 significand. The 36 digit
+// per operand row: 54 bits of the row's largest value, more than an FP64 significand (a value 2^-k of that
+// largest one keeps 54 - k bits: the error is relative to the operand rows' maxima). The 36 digit
 // products of levels s + t <= 7 accumulate exactly in FP32 (products at most 2^12, 8 pairs a level, so
 // 512 entries of K stay below 2^24), the levels combine in integers and round once to FP64. Balanced
 // digits (against 7 unsigned ones, products up to 2^14) are what lets 512 entries of K, not 64, go by
