@@ -110,7 +110,7 @@ __device__ __forceinline__ void drain8(uint32_t taddr, int bE, const int* bF, do
 
 // The combined levels of 8 columns as FP32 pairs: levels 4 to 7 by FP32 Horner steps (they weigh 2^-28 and
 // less), levels 0 to 3 by two-sums, scaled by 2^(E + F - 10). On the FP32 pipe, against the integer pipe of
-// drain8, which the cutting of digits already fills; about 2^-48 of the result.
+// drain8, which the cutting of digits already fills; about 2^-48 of the result and of the largest product.
 __device__ __forceinline__ void drain8_pairs(uint32_t taddr, int bE, const int* bF, float* h, float* l) {
   float v[4][8], lo[8];
   tmem_ld_levels(taddr + 4 * ZN, v);
